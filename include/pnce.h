@@ -52,7 +52,8 @@ typedef enum {
     PNCE_ESTATE = 6         /* wrong device current, or handle/pilot mismatch */
 } pnce_status;
 
-/* Arithmetic of the correlation.  FP32_SIMT: exact FP32 on the CUDA cores.  The others
+/* Arithmetic of the correlation.  FP32_SIMT: FP32 sums of +-y on the CUDA cores (for
+ * m-sequence pilots of 127 <= N <= 16383 by the fast m-sequence transform).  The others
  * quantise Y (per antenna, power-of-two scale) and run on the tensor cores with FP32
  * accumulation; +-1 pilots are exact in every one of these formats (Sec. III-B uses FP16
  * operands).  AUTO lets the library choose from the shape, see pnce_auto_dtype. */
@@ -286,8 +287,9 @@ pnce_status pnce_trace_read(pnce_handle* h, int* kinds, float* ms, int max_entri
  * kl_max, dtype) bytes (0 for invalid shapes).  Enqueues on `stream`, each kernel a
  * programmatic dependent of the one before it: a table / row-map kernel, then for the
  * tensor-core dtypes the quantiser (reading each row from its request's Y), the
- * correlation and a scatter into the requests' H; for FP32 with kl_max > 32 the SIMT
- * correlation reading the rows from the requests' Y (after a row gather into the
+ * correlation and a scatter into the requests' H; for FP32 with an m-sequence pilot the
+ * fast transform, reading from and writing into the requests' buffers; with other pilots
+ * and kl_max > 32 the SIMT correlation reading the rows from the requests' Y (after a row gather into the
  * workspace when kl_max > 256) and writing each row's lags into its request's H; for
  * FP32 with kl_max <= 32 a row gather, the correlation and a scatter.  Allocates nothing.
  */
@@ -422,8 +424,8 @@ pnce_status pnce_estimate_static(pnce_handle* h, const pnce_pilot* pilot, const 
                                  void* stream);
 
 /*
- * Fast m-sequence transform: a yardstick beside the paper's method, not part of it (the
- * paper correlates with the dense circulant, Sec. III-B).  For an m-sequence pilot of
+ * Fast m-sequence transform as an entry point of its own (the paper correlates with the
+ * dense circulant, Sec. III-B; pnce_estimate in FP32 takes the same kernel).  For an m-sequence pilot of
  * degree r (N = 2^r - 1) the same estimate, H[f][m][k][l] = (1/N) sum_n Y[f][m][n]
  * p[(n - l - kL) mod N], is a permutation of each received row into a vector of 2^r
  * entries, a Walsh-Hadamard transform and a gather of the K*L lags: O(N log N) per row

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -257,9 +258,16 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
     // wrapped table: bit t = bit (t mod N) for t < 32 * words, words = ceil(N/32) + 2, so that
     // any 32-bit window starting below N is readable from two consecutive words
     const int words = (N + 31) / 32 + 2;
+    // then, for an m-sequence of a supported degree, the tables of its fast transform, from
+    // the next 16-byte boundary on
+    const size_t bits_bytes = pnce::round_up(sizeof(uint32_t) * (size_t)words, 16);
+    size_t mst_bytes = pnce::mst_table_bytes(N);
     std::vector<uint32_t> ext;
     try {
-        ext.assign((size_t)words, 0u);
+        ext.assign((bits_bytes + mst_bytes) / sizeof(uint32_t), 0u);
+        if (mst_bytes &&
+            !pnce::mst_build_tables(bits_host, N, reinterpret_cast<uint16_t*>(ext.data() + bits_bytes / 4)))
+            mst_bytes = 0;
     } catch (...) {
         return PNCE_ENOMEM;
     }
@@ -273,12 +281,14 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
     p->device = h->device;
     p->N = N;
     p->ext_words = words;
-    if (cudaMalloc(&p->ext_bits_dev, sizeof(uint32_t) * words) != cudaSuccess) {
+    const size_t bytes = bits_bytes + mst_bytes;
+    if (cudaMalloc(&p->ext_bits_dev, bytes) != cudaSuccess) {
         delete p;
         return PNCE_ENOMEM;
     }
-    if (cudaMemcpy(p->ext_bits_dev, ext.data(), sizeof(uint32_t) * words,
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+    const uint16_t* tab = reinterpret_cast<const uint16_t*>(p->ext_bits_dev + bits_bytes / 4);
+    if (cudaMemcpy(p->ext_bits_dev, ext.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+        (mst_bytes && pnce::mst_setup(p->mst, tab, N, h->num_sms, h->max_smem_optin) != cudaSuccess)) {
         cudaFree(p->ext_bits_dev);
         delete p;
         return PNCE_ECUDA;

@@ -20,13 +20,14 @@
 #include <vector>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 struct pnce_fmt {
     int device;
     int N;
     int r;
-    uint16_t* pos_dev;      // s_n, n < N
-    uint16_t* lag_dev;      // u_j, j < N
+    uint16_t* tab_dev;      // r < kMstMinR: s_n (n < N), then u_j (j < N); else mst's tables
+    pnce::MstTables mst;
 };
 
 namespace {
@@ -98,87 +99,6 @@ fmt_kernel(const float2* __restrict__ Y, long long A, int N, int r,
     }
 }
 
-// The same for 2^r >= 512 (r <= 14), laid out to keep shared memory conflict-free: warp w
-// takes segments of 512 consecutive entries, lane l holding entries l + 32 m (m < 16), so
-// the butterfly levels at distances 1..16 are lane exchanges (shuffles) and those at
-// 32..256 stay in the thread's registers; the r - 9 levels at distances 512.. S/2 follow
-// in one more pass over groups of entries 512 apart.  Every shared-memory access of the
-// passes is 32 consecutive entries per warp instruction.
-template <int R>
-__global__ void __launch_bounds__(THREADS, R >= 14 ? 3 : 4)   // 4 rows in flight per SM
-fmt_kernel_seg(const float2* __restrict__ Y, long long A, int N,
-               const uint16_t* __restrict__ pos, const uint16_t* __restrict__ lagvec, int KL,
-               float invN, float2* __restrict__ H) {
-    constexpr int S = 1 << R;
-    constexpr int SEG = 512, NSEG = S / SEG;
-    constexpr int CR = R - 9;                  // levels across segments
-    constexpr int CG = 1 << CR;                // entries per group of the last pass
-    extern __shared__ float2 X[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (long long a = blockIdx.x; a < A; a += gridDim.x) {
-        const float2* y = Y + a * N;
-        if (tid == 0) X[0] = make_float2(0.f, 0.f);
-        for (int n = tid; n < N; n += THREADS) X[__ldg(pos + n)] = __ldcs(y + n);
-        __syncthreads();
-        for (int seg = warp; seg < NSEG; seg += THREADS / 32) {
-            float2* xs = X + seg * SEG + lane;
-            float2 v[16];
-#pragma unroll
-            for (int m = 0; m < 16; ++m) v[m] = xs[32 * m];
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const bool upper = (lane & d) != 0;
-#pragma unroll
-                for (int m = 0; m < 16; ++m) {
-                    const float px = __shfl_xor_sync(0xffffffffu, v[m].x, d);
-                    const float py = __shfl_xor_sync(0xffffffffu, v[m].y, d);
-                    v[m] = upper ? make_float2(px - v[m].x, py - v[m].y)
-                                 : make_float2(v[m].x + px, v[m].y + py);
-                }
-            }
-#pragma unroll
-            for (int dm = 1; dm < 16; dm <<= 1) {
-#pragma unroll
-                for (int m = 0; m < 16; ++m) {
-                    if (m & dm) continue;
-                    const float2 p = v[m], q = v[m + dm];
-                    v[m] = make_float2(p.x + q.x, p.y + q.y);
-                    v[m + dm] = make_float2(p.x - q.x, p.y - q.y);
-                }
-            }
-#pragma unroll
-            for (int m = 0; m < 16; ++m) xs[32 * m] = v[m];
-        }
-        __syncthreads();
-        if constexpr (CR > 0) {
-            for (int g = tid; g < SEG; g += THREADS) {
-                float2 w[CG];
-#pragma unroll
-                for (int k = 0; k < CG; ++k) w[k] = X[g + SEG * k];
-#pragma unroll
-                for (int dk = 1; dk < CG; dk <<= 1) {
-#pragma unroll
-                    for (int k = 0; k < CG; ++k) {
-                        if (k & dk) continue;
-                        const float2 p = w[k], q = w[k + dk];
-                        w[k] = make_float2(p.x + q.x, p.y + q.y);
-                        w[k + dk] = make_float2(p.x - q.x, p.y - q.y);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < CG; ++k) X[g + SEG * k] = w[k];
-            }
-            __syncthreads();
-        }
-        float2* out = H + a * KL;
-        for (int j = tid; j < KL; j += THREADS) {
-            const float2 w = X[__ldg(lagvec + j)];
-            out[j] = make_float2(w.x * invN, w.y * invN);
-        }
-        __syncthreads();   // X is refilled for the next row
-    }
-}
-
 }  // namespace
 
 extern "C" {
@@ -222,14 +142,20 @@ pnce_status pnce_fmt_create(pnce_handle* h, const uint32_t* bits_host, int N, pn
     if (!h || !bits_host || !out) return PNCE_EINVAL;
     *out = nullptr;
     if (N < 3 || (long long)N + 1 > (1LL << MAX_R)) return PNCE_EINVAL;   // before allocating
-    std::vector<uint16_t> pos, lag;
+    size_t bytes = pnce::mst_table_bytes(N);
+    const bool mst = bytes != 0;
+    if (!mst) bytes = sizeof(uint16_t) * 2 * (size_t)N;
+    std::vector<uint16_t> tab;
+    pnce_status st = PNCE_OK;
     try {
-        pos.resize((size_t)N);
-        lag.resize((size_t)N);
+        tab.resize(bytes / sizeof(uint16_t));
+        if (!mst)
+            st = pnce_fmt_tables(bits_host, N, tab.data(), tab.data() + N);
+        else if (!pnce::mst_build_tables(bits_host, N, tab.data()))
+            st = PNCE_EINVAL;
     } catch (...) {
         return PNCE_ENOMEM;
     }
-    pnce_status st = pnce_fmt_tables(bits_host, N, pos.data(), lag.data());
     if (st != PNCE_OK) return st;
     st = on_device(h);
     if (st != PNCE_OK) return st;
@@ -239,18 +165,13 @@ pnce_status pnce_fmt_create(pnce_handle* h, const uint32_t* bits_host, int N, pn
     f->N = N;
     f->r = 0;
     while ((1 << f->r) < N + 1) ++f->r;
-    f->pos_dev = nullptr;
-    f->lag_dev = nullptr;
-    const size_t bytes = sizeof(uint16_t) * (size_t)N;
-    if (cudaMalloc(&f->pos_dev, bytes) != cudaSuccess || cudaMalloc(&f->lag_dev, bytes) != cudaSuccess) {
-        cudaFree(f->pos_dev);
+    if (cudaMalloc(&f->tab_dev, bytes) != cudaSuccess) {
         delete f;
         return PNCE_ENOMEM;
     }
-    if (cudaMemcpy(f->pos_dev, pos.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(f->lag_dev, lag.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
-        cudaFree(f->pos_dev);
-        cudaFree(f->lag_dev);
+    if (cudaMemcpy(f->tab_dev, tab.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+        (mst && pnce::mst_setup(f->mst, f->tab_dev, N, h->num_sms, h->max_smem_optin) != cudaSuccess)) {
+        cudaFree(f->tab_dev);
         delete f;
         return PNCE_ECUDA;
     }
@@ -263,8 +184,7 @@ pnce_status pnce_fmt_destroy(pnce_fmt* f) {
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(f->device);
-    cudaFree(f->pos_dev);
-    cudaFree(f->lag_dev);
+    cudaFree(f->tab_dev);
     if (prev >= 0) cudaSetDevice(prev);
     delete f;
     return PNCE_OK;
@@ -279,36 +199,24 @@ pnce_status pnce_estimate_fmt(pnce_handle* h, const pnce_fmt* f, const void* Y_d
     if (st != PNCE_OK) return st;
     if (f->device != h->device) return PNCE_ESTATE;
     const long long A = (long long)F * M;
-    const size_t smem = sizeof(float2) << f->r;
-    if (f->r < 9 && cudaFuncSetAttribute(fmt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem) != cudaSuccess)
-        return PNCE_ECUDA;
-    const long long grid = A < 0x7fffffffLL ? A : 0x7fffffffLL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float2* Y = static_cast<const float2*>(Y_dev);
     float2* H = static_cast<float2*>(H_dev);
-    const float invN = (float)(1.0 / (double)N);
     pnce::TraceScope tr(h, s, pnce::TRACE_FMT);
-    if (f->r >= 9) {
-        void (*kern)(const float2*, long long, int, const uint16_t*, const uint16_t*, int,
-                     float, float2*) = nullptr;
-        switch (f->r) {
-            case 9: kern = fmt_kernel_seg<9>; break;
-            case 10: kern = fmt_kernel_seg<10>; break;
-            case 11: kern = fmt_kernel_seg<11>; break;
-            case 12: kern = fmt_kernel_seg<12>; break;
-            case 13: kern = fmt_kernel_seg<13>; break;
-            default: kern = fmt_kernel_seg<14>; break;
-        }
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
-            return PNCE_ECUDA;
-        kern<<<(unsigned)grid, THREADS, smem, s>>>(Y, A, N, f->pos_dev, f->lag_dev, K * L, invN,
-                                                   H);
-    } else {
-        fmt_kernel<<<(unsigned)grid, THREADS, smem, s>>>(Y, A, N, f->r, f->pos_dev, f->lag_dev,
-                                                         K * L, invN, H);
+    if (f->mst.tab) {
+        pnce::MstLaunch l;
+        l.Y = Y;
+        l.y_stride = N;
+        l.A = A;
+        l.lags = pnce::lagmap_contiguous(K * L);
+        l.H = H;
+        return pnce::launch_mst(f->mst, l, s) == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
     }
+    const size_t smem = sizeof(float2) << f->r;      // 512 bytes at most
+    const long long grid = A < 0x7fffffffLL ? A : 0x7fffffffLL;
+    const float invN = (float)(1.0 / (double)N);
+    fmt_kernel<<<(unsigned)grid, THREADS, smem, s>>>(Y, A, N, f->r, f->tab_dev, f->tab_dev + N,
+                                                     K * L, invN, H);
     return cudaGetLastError() == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
 }
 

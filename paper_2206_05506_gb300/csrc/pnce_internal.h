@@ -84,11 +84,22 @@ struct TraceScope {
 };
 }  // namespace pnce
 
+namespace pnce {
+// Fast m-sequence transform of one pilot (pnce_mst.cu): its tables on the device (null: the
+// pilot is no m-sequence of a supported degree) and the launch shape that fits an SM.
+struct MstTables {
+    const uint16_t* tab = nullptr;
+    int N = 0, r = 0;
+    int num_sms = 0, block_teams = 0, blocks_per_sm = 0;
+};
+}  // namespace pnce
+
 struct pnce_pilot {
     int device;
     int N;
     int ext_words;                      // words of the wrapped bit table
     uint32_t* ext_bits_dev;             // bit t = pilot bit (t mod N), t < 32 * ext_words
+    pnce::MstTables mst;                // tables in the same allocation, after the bits
 };
 
 namespace pnce {

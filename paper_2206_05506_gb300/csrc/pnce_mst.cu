@@ -1,0 +1,439 @@
+// Correlation with an m-sequence pilot by the fast m-sequence transform, FP32 on the CUDA
+// cores.  For an m-sequence of degree r (N = 2^r - 1) the r-bit windows s_n of the pilot bits
+// run through every nonzero vector once and every bit is a GF(2)-linear function of any
+// window: p[(n - j) mod N] = (-1)^<u_j, s_n>.  So the correlation of Eq. 3 is
+//     N H[j] = W[u_j],   W = Walsh-Hadamard transform of X,  X[s_n] = y[n], X[0] = 0
+// (tables s_n and u_j: pnce_fmt_tables): r levels of additions per row instead of K*L
+// multiply-adds per sample, each output still a sum of +-y.
+//
+// What bounds it: HBM (8 bytes a sample in, 8 a lag out), provided that the shared-memory
+// data path (128 B a clock per SM) is not taken by the two permutations and by moving the
+// vector between the butterfly levels.  Hence:
+//  * Each thread keeps E = 2^LE entries in registers (E = 64 for r >= 11), so that the r
+//    levels take two register passes with one exchange through shared memory between them,
+//    and no lane shuffles (one or two levels of them for r = 7, 13, 14).
+//  * Both permutations are free of bank conflicts.  Sample n is copied (cp.async) to a slot of
+//    the row's buffer that the host has chosen: the 16 slots of line s >> 4 hold the 16
+//    entries that a half-warp reads together, in an order such that the 16 consecutive
+//    samples that a half-warp writes together also lie in 16 different bank pairs.  Such an
+//    order exists for any permutation (the entries are the edges of a 16-regular bipartite
+//    multigraph between write groups and read groups, which 16 colours colour properly) and
+//    is found by four halvings of the graph.  The same on the way out.  Addressed by s itself,
+//    the scatter and the gather each took about 3 wavefronts for every one they need.
+//    (With the r <= 8 levels of a pass done by lane shuffles and X addressed by s, 512 frames x
+//    128 rows of N = 4095 with 2048 lags took 0.93 ms; now 0.67 ms, 4.8 TB/s.)
+//  * A team of G = 2^r / E threads (one warp or less for r <= 11) owns a row; teams only
+//    synchronise within themselves, so the rows of an SM sit in different phases and the
+//    loads of some overlap the additions of others.
+// Against the dense sum (pnce_simt.cu): N = 4095, 2048 lags, 65536 rows 34.4 -> 0.67 ms;
+// N = 1023, 512 lags, 8192 rows 0.283 -> 0.028 ms; and closer to the 64-bit result (relative
+// error 0.7-1.0e-7 where the dense sum has 5e-7-1.1e-6: fewer roundings per output).
+#include <new>
+#include <vector>
+
+#include "pnce_mst.h"
+
+namespace {
+
+// Entries per thread for degree r
+constexpr int mst_le(int r) {
+    return r >= 11 ? 6 : r >= 9 ? 5 : r == 8 ? 4 : 3;
+}
+
+template <int R>
+struct Mst {
+    static constexpr int LE = mst_le(R), E = 1 << LE;
+    static constexpr int LG = R - LE, G = 1 << LG;       // threads per row
+    static constexpr int L2 = LG < LE ? LG : LE;         // levels of the second register pass
+    static constexpr int X = LG > LE ? LG - LE : 0;      // levels by lane shuffles
+    static constexpr int S = 1 << R;
+    static constexpr int TEAM = G < 32 ? 32 : G;         // threads that synchronise
+    static constexpr int RT = TEAM / G;                  // rows per team
+    static constexpr int ROW = S + (S >> L2);            // entries of a row's buffer, padded
+    // tables in shared memory; for r >= 13 they are read from global memory
+    static constexpr bool TAB_SMEM = R <= 12;
+    static constexpr int TAB = TAB_SMEM ? S * 6 + S / 2 : 0;
+    // most threads per block and most blocks per SM (registers: 2 E + about 40 each)
+    static constexpr int MAXT = R >= 14 ? 256 : R >= 11 ? 384 : R >= 9 ? 640 : 512;
+    static constexpr int MINB = R >= 9 ? 1 : 2;
+    static constexpr size_t team_bytes() { return (size_t)RT * ROW * sizeof(float2); }
+};
+
+// entry of register k of thread t in the second pass
+__host__ __device__ constexpr int pass2_entry(int le, int lg, int t, int k) {
+    return lg <= le ? ((t + ((k >> lg) << lg)) << lg) | (k & ((1 << lg) - 1))
+                    : (t << le) | k;
+}
+
+template <int TEAM>
+__device__ __forceinline__ void team_sync(int team) {
+    if constexpr (TEAM <= 32)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(TEAM) : "memory");
+}
+
+__device__ __forceinline__ void cp_async8(unsigned smem, const void* gmem, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem), "l"(gmem),
+                 "r"(bytes)
+                 : "memory");
+}
+
+// butterfly levels on register distances FIRST, 2 FIRST, .. < LAST
+template <int E, int FIRST, int LAST>
+__device__ __forceinline__ void butterflies(float2 (&v)[E]) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+#pragma unroll
+    for (int d = FIRST; d < LAST; d <<= 1) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            if (k & d) continue;
+            const float2 a = v[k], b = v[k + d];
+            v[k] = __fadd2_rn(a, b);
+            v[k + d] = __ffma2_rn(b, m1, a);       // a - b, rounded once
+        }
+    }
+}
+
+template <int R, bool GRP>
+__global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
+mst_kernel(const pnce::MstLaunch p) {
+    using M = Mst<R>;
+    constexpr int E = M::E, G = M::G, LG = M::LG, LE = M::LE, S = M::S;
+    extern __shared__ __align__(16) unsigned char mst_smem[];
+    const int tid = threadIdx.x;
+    const uint16_t* tab;
+    if constexpr (M::TAB_SMEM) {
+        const uint4* src = reinterpret_cast<const uint4*>(p.tab);
+        uint4* dst = reinterpret_cast<uint4*>(mst_smem);
+        for (int i = tid; i < M::TAB / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+        tab = reinterpret_cast<const uint16_t*>(mst_smem);
+        __syncthreads();
+    } else {
+        tab = p.tab;
+    }
+    const uint4* in_slot = reinterpret_cast<const uint4*>(tab);            // [E/8][G] x 8
+    const uint4* out_slot = reinterpret_cast<const uint4*>(tab + S);       // [E/8][G] x 8
+    const uint16_t* lag_slot = tab + 2 * S;                                // [N]
+    const uint32_t* in_col = reinterpret_cast<const uint32_t*>(tab + 3 * S);   // [E/8][G]
+
+    // as a programmatic dependent the tables came in beside the kernel before; the row map
+    // and the rows are read only after it has finished
+    if constexpr (GRP) asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    const int team = tid / M::TEAM, t = tid % G, sub = (tid % M::TEAM) / G;
+    float2* buf = reinterpret_cast<float2*>(mst_smem + M::TAB) + (team * M::RT + sub) * M::ROW;
+    const unsigned sbuf = (unsigned)__cvta_generic_to_shared(buf);
+    const int teams = blockDim.x / M::TEAM;
+    const long long stride = (long long)gridDim.x * teams * M::RT;
+
+    for (long long row0 = ((long long)blockIdx.x * teams + team) * M::RT; row0 < p.A;
+         row0 += stride) {
+        const long long row = row0 + sub;
+        const float2* y = nullptr;
+        float2* h = nullptr;
+        int cols = p.lags.ldH;
+        if (row < p.A) {
+            if constexpr (GRP) {
+                const int b = __ldg(p.row_req + row);
+                if (b >= 0) {
+                    const pnce_req_desc& q = p.dd[b];
+                    cols = q.K * q.L;
+                    y = static_cast<const float2*>(q.Y) + (row - q.row_offset) * p.N;
+                    h = static_cast<float2*>(q.H) + (row - q.row_offset) * cols;
+                }
+            } else {
+                y = p.Y + row * p.y_stride;
+                h = p.H + row * p.lags.ldH;
+            }
+        }
+        if constexpr (GRP) {                       // a team without a row has nothing to do
+            if (M::RT == 1 ? y == nullptr : __all_sync(0xffffffffu, y == nullptr)) continue;
+        }
+        if (y) {
+#pragma unroll
+            for (int i8 = 0; i8 < E / 8; ++i8) {
+                const uint4 q = in_slot[i8 * G + t];
+                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int n = t + G * (8 * i8 + e);
+                    const unsigned slot = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu;
+                    const bool ok = 8 * i8 + e < E - 1 || n < p.N;     // entry 0 of X is zero
+                    cp_async8(sbuf + 8 * slot, ok ? y + n : y, ok ? 8 : 0);
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        team_sync<M::TEAM>(team);
+
+        float2 v[E];
+        // first pass: register k holds entry k G + t, levels G .. S/2
+#pragma unroll
+        for (int k8 = 0; k8 < E / 8; ++k8) {
+            const uint32_t c = in_col[k8 * G + t];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int k = 8 * k8 + e;
+                v[k] = buf[k * G + (t & ~15) + ((c >> (4 * e)) & 15u)];
+            }
+        }
+        butterflies<E, 1, E>(v);
+        team_sync<M::TEAM>(team);                  // the buffer is read: reuse it
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int s = k * G + t;
+            buf[s + (s >> M::L2)] = v[k];
+        }
+        team_sync<M::TEAM>(team);
+        // second pass: the low L2 levels in registers, the X above them by lane shuffles
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int s = pass2_entry(LE, LG, t, k);
+            v[k] = buf[s + (s >> M::L2)];
+        }
+        butterflies<E, 1, (1 << M::L2)>(v);
+        if constexpr (M::X > 0) {
+#pragma unroll
+            for (int d = 1; d < (1 << M::X); d <<= 1) {
+                const float sg = (t & d) ? -1.f : 1.f;
+#pragma unroll
+                for (int k = 0; k < E; ++k) {
+                    const float px = __shfl_xor_sync(0xffffffffu, v[k].x, d);
+                    const float py = __shfl_xor_sync(0xffffffffu, v[k].y, d);
+                    v[k] = make_float2(fmaf(sg, v[k].x, px), fmaf(sg, v[k].y, py));
+                }
+            }
+        }
+        team_sync<M::TEAM>(team);
+        // out: only the lines of lags that are wanted (contiguous lags), all of them otherwise
+        const unsigned lim = p.lags.mode == 0 ? (unsigned)((cols + 15) & ~15) : (unsigned)S;
+#pragma unroll
+        for (int k8 = 0; k8 < E / 8; ++k8) {
+            const uint4 q = out_slot[k8 * G + t];
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const unsigned slot = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu;
+                if (slot < lim) buf[slot] = v[8 * k8 + e];
+            }
+        }
+        team_sync<M::TEAM>(team);
+        if (h) {
+            for (int c = t; c < cols; c += G) {
+                int lag = c;
+                if (!GRP && p.lags.mode != 0) {     // column k L + l holds lag k step + l
+                    const int k = (int)__umulhi((unsigned)c << 4, p.magic_L);
+                    lag = k * p.lags.step + (c - k * p.lags.L);
+                }
+                const float2 w = buf[lag_slot[lag]];
+                h[c] = make_float2(w.x * p.invN, w.y * p.invN);
+            }
+        }
+        team_sync<M::TEAM>(team);                  // the buffer takes the next row
+    }
+}
+
+template <int R>
+cudaError_t launch_r(const pnce::MstTables& m, const pnce::MstLaunch& p, cudaStream_t s) {
+    using M = Mst<R>;
+    // rows spread over the SMs first, then over the teams of a block
+    const long long teams = (p.A + M::RT - 1) / M::RT;
+    const long long sms = m.num_sms;
+    const int max_teams = m.block_teams;
+    long long per = (teams + sms - 1) / sms;
+    if (per > max_teams) per = max_teams;
+    long long grid = (teams + per - 1) / per;
+    const long long resident = sms * (per == max_teams ? m.blocks_per_sm : 1);
+    if (grid > resident) grid = resident;
+    const size_t smem = M::TAB + (size_t)per * M::team_bytes();
+    const unsigned block = (unsigned)(per * M::TEAM);
+    const bool grp = p.dd != nullptr;
+    if (p.pdl) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid, 1, 1);
+        cfg.blockDim = dim3(block, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return grp ? cudaLaunchKernelEx(&cfg, mst_kernel<R, true>, p)
+                   : cudaLaunchKernelEx(&cfg, mst_kernel<R, false>, p);
+    }
+    if (grp)
+        mst_kernel<R, true><<<(unsigned)grid, block, smem, s>>>(p);
+    else
+        mst_kernel<R, false><<<(unsigned)grid, block, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+// Shared-memory limits of both kernels, and how many teams fit an SM.
+template <int R>
+cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
+    using M = Mst<R>;
+    int teams = M::MAXT / M::TEAM;
+    const int fit = (int)((max_smem_optin - M::TAB) / M::team_bytes());
+    if (fit < 1) return cudaErrorNotSupported;
+    if (teams > fit) teams = fit;
+    const int smem = M::TAB + teams * (int)M::team_bytes();
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(mst_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  smem)) != cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(mst_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  smem)) != cudaSuccess)
+        return e;
+    m.block_teams = teams;
+    int per = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mst_kernel<R, false>,
+                                                           teams * M::TEAM, smem)) != cudaSuccess)
+        return e;
+    m.blocks_per_sm = per < 1 ? 1 : per;
+    return cudaSuccess;
+}
+
+// Proper 16-colouring of a 16-regular bipartite multigraph given as edges (l[e], r[e]),
+// e < S, both sides of S / 16 vertices: four times, the edges of a class are split into two
+// classes of half the degree by pairing them up at every vertex and colouring the cycles that
+// the pairs form alternately.
+void colour16(const std::vector<int>& l, const std::vector<int>& r, std::vector<uint8_t>& col) {
+    const int S = (int)l.size(), V = S / 16;
+    col.assign((size_t)S, 0);
+    std::vector<int> pl((size_t)S), pr((size_t)S), open((size_t)V * 16);
+    std::vector<int8_t> half((size_t)S);
+    for (int level = 0; level < 4; ++level) {
+        for (int side = 0; side < 2; ++side) {
+            const std::vector<int>& v = side ? r : l;
+            std::vector<int>& p = side ? pr : pl;
+            std::fill(open.begin(), open.end(), -1);
+            for (int e = 0; e < S; ++e) {
+                int& o = open[(size_t)v[(size_t)e] * 16 + col[(size_t)e]];
+                if (o < 0) {
+                    o = e;
+                } else {
+                    p[(size_t)e] = o;
+                    p[(size_t)o] = e;
+                    o = -1;
+                }
+            }
+        }
+        std::fill(half.begin(), half.end(), (int8_t)-1);
+        for (int e0 = 0; e0 < S; ++e0)
+            for (int e = e0; half[(size_t)e] < 0; e = pr[(size_t)pl[(size_t)e]]) {
+                half[(size_t)e] = 0;
+                half[(size_t)pl[(size_t)e]] = 1;
+            }
+        for (int e = 0; e < S; ++e)
+            col[(size_t)e] = (uint8_t)(2 * col[(size_t)e] + half[(size_t)e]);
+    }
+}
+
+}  // namespace
+
+namespace pnce {
+
+size_t mst_table_bytes(int N) {
+    int r = 0;
+    while ((1LL << r) < (long long)N + 1) ++r;
+    if ((1LL << r) != (long long)N + 1 || r < kMstMinR || r > kMstMaxR) return 0;
+    return (size_t)(N + 1) * 13 / 2;
+}
+
+bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out) {
+    if (mst_table_bytes(N) == 0) return false;
+    int r = 0;
+    while ((1 << r) < N + 1) ++r;
+    const int S = 1 << r, le = mst_le(r), lg = r - le, E = 1 << le, G = 1 << lg;
+    std::vector<uint16_t> pos((size_t)N), lag((size_t)N);
+    if (pnce_fmt_tables(bits_host, N, pos.data(), lag.data()) != PNCE_OK) return false;
+    std::vector<int> l((size_t)S), rr((size_t)S), of((size_t)S);
+    std::vector<uint8_t> col;
+    uint16_t* in_slot = out;
+    uint16_t* out_slot = out + S;
+    uint16_t* lag_slot = out + 2 * S;
+    uint8_t* in_col = reinterpret_cast<uint8_t*>(out + 3 * S);
+    // in: edge n joins write group n >> 4 to read group s_n >> 4 (n = N: entry 0)
+    for (int n = 0; n < S; ++n) {
+        const int s = n < N ? pos[(size_t)n] : 0;
+        l[(size_t)n] = n >> 4;
+        rr[(size_t)n] = s >> 4;
+    }
+    colour16(l, rr, col);
+    for (int n = 0; n < S; ++n) {
+        const int s = n < N ? pos[(size_t)n] : 0;
+        const int i = n / G, t = n % G;
+        in_slot[((i / 8) * G + t) * 8 + i % 8] = (uint16_t)((s & ~15) | col[(size_t)n]);
+        of[(size_t)s] = col[(size_t)n];
+    }
+    for (int t = 0; t < G; ++t)
+        for (int k = 0; k < E; k += 2)
+            in_col[4 * ((k / 8) * G + t) + (k % 8) / 2] =
+                (uint8_t)(of[(size_t)(k * G + t)] | (of[(size_t)((k + 1) * G + t)] << 4));
+    // out: edge j joins the half-warp that holds entry u_j to read group j >> 4
+    std::vector<int> half_of((size_t)S);
+    for (int t = 0; t < G; ++t)
+        for (int k = 0; k < E; ++k)
+            half_of[(size_t)pass2_entry(le, lg, t, k)] = k * (G / 16) + (t >> 4);
+    std::fill(of.begin(), of.end(), N);                       // lag of an entry (0: none)
+    for (int j = 0; j < N; ++j) of[lag[(size_t)j]] = j;
+    for (int j = 0; j < S; ++j) {
+        l[(size_t)j] = half_of[j < N ? lag[(size_t)j] : 0];
+        rr[(size_t)j] = j >> 4;
+    }
+    colour16(l, rr, col);
+    for (int j = 0; j < S; ++j) lag_slot[j] = (uint16_t)((j & ~15) | col[(size_t)j]);
+    for (int t = 0; t < G; ++t)
+        for (int k = 0; k < E; ++k)
+            out_slot[((k / 8) * G + t) * 8 + k % 8] =
+                lag_slot[of[(size_t)pass2_entry(le, lg, t, k)]];
+    return true;
+}
+
+cudaError_t mst_setup(MstTables& m, const uint16_t* tab_dev, int N, int num_sms,
+                      int max_smem_optin) {
+    m.tab = nullptr;
+    m.N = N;
+    m.num_sms = num_sms;
+    m.r = 0;
+    while ((1 << m.r) < N + 1) ++m.r;
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (m.r) {
+        case 7: e = setup_r<7>(m, max_smem_optin); break;
+        case 8: e = setup_r<8>(m, max_smem_optin); break;
+        case 9: e = setup_r<9>(m, max_smem_optin); break;
+        case 10: e = setup_r<10>(m, max_smem_optin); break;
+        case 11: e = setup_r<11>(m, max_smem_optin); break;
+        case 12: e = setup_r<12>(m, max_smem_optin); break;
+        case 13: e = setup_r<13>(m, max_smem_optin); break;
+        case 14: e = setup_r<14>(m, max_smem_optin); break;
+        default: break;
+    }
+    if (e == cudaSuccess) m.tab = tab_dev;
+    return e;
+}
+
+cudaError_t launch_mst(const MstTables& m, MstLaunch p, cudaStream_t s) {
+    if (p.A <= 0) return cudaSuccess;
+    p.tab = m.tab;
+    p.N = m.N;
+    p.invN = (float)(1.0 / (double)m.N);
+    // c / L for c < 2^14 and L < 2^14 as the high word of 16 c * magic_L
+    p.magic_L = p.lags.mode ? (unsigned)(((1u << 28) + (unsigned)p.lags.L - 1) / (unsigned)p.lags.L)
+                            : 0u;
+    switch (m.r) {
+        case 7: return launch_r<7>(m, p, s);
+        case 8: return launch_r<8>(m, p, s);
+        case 9: return launch_r<9>(m, p, s);
+        case 10: return launch_r<10>(m, p, s);
+        case 11: return launch_r<11>(m, p, s);
+        case 12: return launch_r<12>(m, p, s);
+        case 13: return launch_r<13>(m, p, s);
+        case 14: return launch_r<14>(m, p, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace pnce

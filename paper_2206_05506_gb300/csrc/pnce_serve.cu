@@ -11,6 +11,7 @@
 // GB300: 2.15 GB in and 1.07 GB out together in 10.6 ms against 11.3 ms with two DMAs; the
 // inbound copy alone takes 10.15 ms).
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -242,6 +243,16 @@ pnce_status pnce_estimate_grouped(pnce_handle* h, const pnce_pilot* pilot,
                                                    h->status_dev);
     if (cudaGetLastError() != cudaSuccess) return PNCE_ECUDA;
     if (dtype == PNCE_FP32_SIMT) {
+        if (pilot->mst.tab) {
+            pnce::MstLaunch l;
+            l.A = rows;
+            l.lags = pnce::lagmap_contiguous(kl_max);
+            l.dd = dd;
+            l.row_req = row_req;
+            l.pdl = !h->trace_on;
+            pnce::TraceScope tr(h, s, pnce::TRACE_SIMT);
+            return pnce::launch_mst(pilot->mst, l, s) == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
+        }
         float2* Yb = reinterpret_cast<float2*>(ws + lay.y_off);
         if (pnce::simt_grouped_ok(N, kl_max)) {
             // the SIMT kernel writes each row's lags into its request; it reads the rows

@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -652,9 +653,7 @@ namespace pnce {
 
 cudaError_t launch_simt_bits(const pnce_pilot* pilot, const float2* Y, long long A, int N,
                              int KL, float2* H, cudaStream_t s) {
-    if (KL <= FEW_LAGS) return launch_few_lags(pilot->ext_bits_dev, Y, N, A, N, KL, KL, H, s);
-    return launch<FWD_BITS>(pilot->ext_bits_dev, nullptr, Y, N, A, N, lagmap_contiguous(KL), N,
-                            H, s);
+    return launch_simt_bits_ex(pilot, Y, N, A, N, lagmap_contiguous(KL), H, s);
 }
 
 bool simt_grouped_ok(int N, int kl_max) { return kl_max > FEW_LAGS && win_len(N) <= WIN_MAX; }
@@ -675,6 +674,15 @@ cudaError_t launch_simt_grouped(const pnce_pilot* pilot, const pnce_req_desc* dd
 cudaError_t launch_simt_bits_ex(const pnce_pilot* pilot, const float2* Y, long long y_stride,
                                 long long A, int N, const LagMap& lags, float2* H,
                                 cudaStream_t s) {
+    if (pilot->mst.tab && !(lags.mode == 0 && lags.ldH <= FEW_LAGS)) {
+        MstLaunch l;
+        l.Y = Y;
+        l.y_stride = y_stride;
+        l.A = A;
+        l.lags = lags;
+        l.H = H;
+        return launch_mst(pilot->mst, l, s);
+    }
     if (lags.mode == 0 && lags.ldH <= FEW_LAGS)
         return launch_few_lags(pilot->ext_bits_dev, Y, y_stride, A, N, lags.ldH, lags.ldH, H, s);
     return launch<FWD_BITS>(pilot->ext_bits_dev, nullptr, Y, y_stride, A, N, lags, N, H, s);

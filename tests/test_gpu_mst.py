@@ -1,0 +1,103 @@
+"""FP32 estimates of m-sequence pilots take the fast transform kernel: against the FP64 oracle
+for every degree it takes, at the edges of its row teams (one row, a half-filled team, more
+rows than fit the GPU at once), the smallest and the largest lag counts it gets, rows with a
+prefix and spread shifts; samples that are not numbers; a pilot with one bit flipped, which
+keeps the dense kernel.
+
+Tolerance: every output is a sum of N terms +-y over r levels of additions, each rounded to
+2^-24 of a partial sum: relative 2-norm error at most about r 2^-24, NMSE (14 2^-24)^2 = 7e-13;
+1e-11 leaves room for partial sums that exceed the result."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import pn_oracle as O
+from synth import mseq
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-11
+
+
+def _y(rng, *shape):
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+
+@pytest.mark.parametrize("A, KL", [(1, 33), (2, -1), (3, 40), (37, 64)])
+@pytest.mark.parametrize("r", range(7, 15))
+def test_fp32_transform_matches_oracle(r, A, KL):
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 1)
+    N = bits.size
+    KL = N if KL < 0 else KL
+    rng = np.random.default_rng([r, A])
+    cp = 5 if A == 37 else 0
+    Y = _y(rng, 1, A, N + cp)
+    pilot = pk.Pilot(bits, device=dev)
+    Yd = torch.from_numpy(Y).to(dev)
+    buf = torch.full((A * KL + 64,), complex(3.0, 3.0), dtype=torch.complex64, device=dev)
+    H = buf[32:32 + A * KL].view(1, A, 1, KL)
+    pk.estimate(Yd, pilot, 1, KL, dtype="fp32", out=H, cp_len=cp)
+    ref = O.estimate_fft(Y[..., cp:], bits, 1, KL)
+    assert O.nmse(H.cpu().numpy(), ref) <= TOL
+    g = torch.cat([buf[:32], buf[-32:]])
+    assert bool((g == complex(3.0, 3.0)).all()), "write outside H"
+    if A == 37:                                   # spread shifts, several transmitters
+        H = pk.estimate(Yd, pilot, 3, 21, dtype="fp32", cp_len=cp, shift_rule="spread")
+        ref = O.estimate_general(Y, bits, 3, 21, cp_len=cp, shifts=np.arange(3) * (N // 3))
+        assert O.nmse(H.cpu().numpy(), ref) <= TOL
+
+
+@pytest.mark.parametrize("r, A", [(7, 20011), (8, 12001), (9, 8003), (10, 4001), (11, 2003), (12, 1009)])
+def test_rows_beyond_one_wave(r, A):
+    # every row alone gives the bits it gives in the batch, on a sample of the rows
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 0)
+    N, KL = bits.size, 50
+    gen = torch.Generator(dev).manual_seed(r)
+    Y = torch.randn(1, A, N, dtype=torch.complex64, device=dev, generator=gen)
+    pilot = pk.Pilot(bits, device=dev)
+    H = pk.estimate(Y, pilot, 1, KL, dtype="fp32")
+    rows = [0, 1, A // 2, A - 2, A - 1]
+    ref = O.estimate(Y[:, rows].cpu().numpy(), bits, 1, KL)
+    assert O.nmse(H[:, rows].cpu().numpy(), ref) <= TOL
+    for a in rows:
+        assert torch.equal(pk.estimate(Y[:, a:a + 1].clone(), pilot, 1, KL, dtype="fp32"), H[:, a:a + 1])
+
+
+@pytest.mark.parametrize("r", [7, 10, 12])
+def test_samples_that_are_not_numbers(r):
+    # as in the sum that defines the estimate: a NaN reaches every lag of its part, an
+    # infinity takes the pilot's sign at every lag, opposite infinities give NaN
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 0)
+    N, KL = bits.size, 70
+    Y = _y(np.random.default_rng(r), 1, 5, N)
+    Y[0, 0, 3] = complex(np.nan, 1.0)
+    Y[0, 1, 4] = complex(2.0, np.inf)
+    Y[0, 2, N - 1] = complex(-np.inf, 0.5)
+    Y[0, 3, [5, 9]] = complex(np.inf, 1.0)
+    H = pk.estimate(torch.from_numpy(Y).to(dev), pk.Pilot(bits, device=dev), 1, KL,
+                    dtype="fp32").cpu().numpy()[0, :, 0]
+    p = 1.0 - 2.0 * bits
+    P = np.stack([np.roll(p, j) for j in range(KL)], axis=1)
+    with np.errstate(invalid="ignore"):
+        want = np.stack([(Y[0].real[:, :, None] * P).sum(1), (Y[0].imag[:, :, None] * P).sum(1)])
+    for got, w in ((H.real, want[0]), (H.imag, want[1])):
+        assert np.array_equal(np.isnan(got), np.isnan(w))
+        inf = np.isinf(w)
+        assert np.array_equal(np.isinf(got), inf) and np.array_equal(np.sign(got[inf]), np.sign(w[inf]))
+        fine = np.isfinite(w)
+        assert np.allclose(got[fine], w[fine] / N, rtol=0, atol=1e-5)
+
+
+def test_other_bits_keep_the_dense_kernel():
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(10, 0).copy()
+    bits[100] ^= 1
+    Y = _y(np.random.default_rng(3), 2, 9, bits.size)
+    H = pk.estimate(torch.from_numpy(Y).to(dev), pk.Pilot(bits, device=dev), 2, 64, dtype="fp32")
+    assert O.nmse(H.cpu().numpy(), O.estimate(Y, bits, 2, 64)) <= TOL
