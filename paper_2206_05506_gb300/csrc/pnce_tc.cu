@@ -283,6 +283,14 @@ __device__ __forceinline__ void tmem_ld16x256b_x8(uint32_t taddr, uint32_t (&v)[
           "=r"(v[31])
         : "r"(taddr));
 }
+__device__ __forceinline__ void red_add4(float2* p, float4 v) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void red_add2(float2* p, float x, float y) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -306,7 +314,7 @@ __device__ __forceinline__ void drain_accumulator(uint32_t tacc, int q, int lane
                                                   float2* __restrict__ H, long long A, int ldH,
                                                   int BN, int col0, int valid,
                                                   long long spacing, int c_lo, int c_hi,
-                                                  Release release) {
+                                                  Release release, bool add = false) {
     const long long c0 = clock64();
     const int g = lane >> 2, u4 = lane & 3;
     long long ant[2];
@@ -342,7 +350,14 @@ __device__ __forceinline__ void drain_accumulator(uint32_t tacc, int q, int lane
                 const float4 val = make_float4(
                     __uint_as_float(v[h][4 * x + 1]) * rs[h], __uint_as_float(v[h][4 * x + 3]) * rs[h],
                     __uint_as_float(v[h][4 * x]) * rs[h], __uint_as_float(v[h][4 * x + 2]) * rs[h]);
-                if (j + 1 < valid && (off & 1) == 0) {
+                if (add) {                  // this thread has stored the first part there
+                    if (j + 1 < valid && (off & 1) == 0) {
+                        red_add4(row + j, val);
+                    } else {
+                        red_add2(row + j, val.x, val.y);
+                        if (j + 1 < valid) red_add2(row + j + 1, val.z, val.w);
+                    }
+                } else if (j + 1 < valid && (off & 1) == 0) {
                     *reinterpret_cast<float4*>(row + j) = val;
                 } else {
                     row[j] = make_float2(val.x, val.y);
@@ -794,6 +809,11 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
     constexpr int a_stage = KPS * A_BOX;        // prm.a_stage
     const uint32_t rank = cluster_rank();
     const long long pair = cluster_id(), npairs = cluster_count();
+    // A tile whose reduction has more than 32 K blocks is summed in two halves, the second
+    // added to the first in FP32 by the epilogue: the tensor cores truncate the accumulator
+    // at every MMA, so half as many MMAs on half the sum lose less (N = 4095, fp16, relative
+    // to 64 bits: 1.4e-6 in one piece).
+    const int halves = num_st * KPS > 32 ? 2 : 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < nst; ++s) {
@@ -883,11 +903,14 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
             unsigned long long* last_bar = nullptr;
             uint32_t last_par = 0;
             bool ok = true;
-            for (long long t = pair; t < prm.num_tiles && ok; t += npairs) {
+            for (long long it = pair * halves; it < prm.num_tiles * halves && ok;
+                 it += (it % halves == halves - 1) ? (npairs - 1) * halves + 1 : 1) {
+                const int st0 = (it % halves) ? num_st / 2 : 0;
+                const int st1 = (it % halves) == halves - 1 ? num_st : num_st / 2;
                 if (!wait_bar<true>(&ctl->tempty[acc], acc_phase ^ 1u, wctl, prm, true)) break;
                 fence_after();
                 const uint32_t d = tmem + acc * ACC_COLS;
-                for (int st = 0; st < num_st; ++st) {
+                for (int st = st0; st < st1; ++st) {
                     if (!wait_bar<true>(&ctl->full_a[stage], phase, wctl, prm, true)) {
                         ok = false;
                         break;
@@ -903,7 +926,7 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
                             umma_pair<DT>(d, ad + (uint64_t)(h * (A_BOX >> 4)) + 2u * ks,
                                           bd + (uint64_t)(h * 8 * F::TS * (F::BK / F::EPR)) +
                                               (KSTEP_B >> 4) * ks,
-                                          idesc, (st | h | ks) != 0);
+                                          idesc, ((st - st0) | h | ks) != 0);
                     umma_commit_pair(&ctl->empty[stage]);
                     last_bar = &ctl->empty[stage];
                     last_par = phase;
@@ -922,7 +945,10 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
         // ------------------------------------------------------ epilogue (both CTAs)
         const int q = warp & 3;
         uint32_t acc = 0, acc_phase = 0;
-        for (long long t = pair; t < prm.num_tiles; t += npairs) {
+        for (long long it = pair * halves; it < prm.num_tiles * halves;
+             it += (it % halves == halves - 1) ? (npairs - 1) * halves + 1 : 1) {
+            const long long t = it / halves;
+            const bool second = it % halves != 0;
             const long long rb = 2 * (t / num_jt) + rank;
             long long j0;
             int col0, valid;
@@ -934,7 +960,7 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
             fence_after();
             unsigned long long* te = &ctl->tempty[acc];
             drain_accumulator(tmem + acc * ACC_COLS, q, lane, rb * (BM / 2), row_scale, H,
-                              prm.A, prm.lags.ldH, BN, col0, valid, prm.epi_spacing, 0,
+                              prm.A, prm.lags.ldH, BN, col0, valid, prm.epi_spacing / halves, 0,
                               (BN + 63) / 64, [&] {
                                   fence_before();
                                   __syncwarp();
@@ -942,7 +968,8 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, const uint32_t* __restr
                                       if (rank == 0) mbar_arrive(te);
                                       else mbar_arrive_remote(te, 0);
                                   }
-                              });
+                              },
+                              second);
             acc ^= 1u;
             if (acc == 0) acc_phase ^= 1u;
         }
