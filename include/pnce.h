@@ -54,8 +54,11 @@ typedef enum {
 
 /* Arithmetic of the correlation.  FP32_SIMT: FP32 sums of +-y on the CUDA cores (for
  * m-sequence pilots of 127 <= N <= 16383 by the fast m-sequence transform).  The others
- * quantise Y (per antenna, power-of-two scale) and run on the tensor cores with FP32
- * accumulation; +-1 pilots are exact in every one of these formats (Sec. III-B uses FP16
+ * quantise Y (per antenna, power-of-two scale) and sum the quantised samples with FP32
+ * accumulation: on the tensor cores, or, for the same m-sequence pilots, by the same
+ * transform in FP32, which is faster and closer to the exact sum (the environment variable
+ * PNCE_TC_FORCE, or any of the switches that pick a tensor-core kernel, keeps the tensor
+ * cores); +-1 pilots are exact in every one of these formats (Sec. III-B uses FP16
  * operands).  AUTO lets the library choose from the shape, see pnce_auto_dtype. */
 typedef enum {
     PNCE_FP32_SIMT = 0,
@@ -116,9 +119,10 @@ size_t pnce_workspace_size(int F, int M, int N, int K, int L, int dtype);
 /*
  * Channel estimate, Eq. 3 / Eq. 10 (definition at the top of this file).
  * Y_dev: complex64 [F][M][N]; H_dev: complex64 [F][M][K][L] (fully overwritten).
- * dtype: a pnce_dtype.  For the tensor-core dtypes Y is first quantised per antenna
- * (pnce_quantize) into workspace_dev, then correlated on the tensor cores; the FP32 SIMT
- * path ignores the workspace (may be NULL).  With the environment variable
+ * dtype: a pnce_dtype.  For the tensor-core dtypes Y is first quantised per antenna as
+ * pnce_quantize does and then correlated, in one launch (m-sequence pilots) or through
+ * workspace_dev, whose contents are unspecified afterwards; the FP32 SIMT path ignores the
+ * workspace (may be NULL).  With the environment variable
  * PNCE_OVERLAP_CHUNKS=n (2..8), a large tensor-core batch is cut into n frame chunks whose
  * quantisation overlaps the previous chunk's correlation on the handle's own streams
  * (the call still behaves as if enqueued on `stream`); by default the two run in order.
@@ -175,9 +179,8 @@ pnce_status pnce_quantize(pnce_handle* h, const void* Y_dev, int F, int M, int N
                           double* power_dev, void* stream);
 
 /*
- * Tensor-core correlation of an operand already quantised into workspace_dev by
- * pnce_quantize (same F, M, N, dtype): the contraction and epilogue of pnce_estimate
- * alone.  Lets callers time or overlap the quantisation separately.
+ * Correlation of an operand already quantised into workspace_dev by pnce_quantize (same F,
+ * M, N, dtype): the second step of pnce_estimate alone, with the same bits.  Lets callers time or overlap the quantisation separately.
  */
 pnce_status pnce_correlate_quantized(pnce_handle* h, const pnce_pilot* pilot,
                                      int F, int M, int N, int K, int L, int dtype,
@@ -246,6 +249,8 @@ pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const vo
  * "pnce.<kind>" (always on; a no-op unless a profiler is attached).
  * pnce_trace_enable creates the events on first use (allocates host and event resources,
  * not device memory) and clears the record; pnce_trace_read waits for the recorded kernels,
+ * (traced calls quantise and correlate in two launches even where an untraced one takes
+ * one; the results are the same bits)
  * returns up to max_entries (kind, milliseconds) pairs -- kind 0 quantiser, 1 tensor-core
  * correlation, 2 FP32 SIMT correlation, 3 fast m-sequence transform, 4 adjoint (dY and
  * dp together) -- in launch order, and

@@ -377,6 +377,12 @@ pnce_status pnce_estimate(pnce_handle* h, const pnce_pilot* pilot, const void* Y
     if (!(h->cc_major == 10 && h->cc_minor == 3)) return PNCE_EUNSUPPORTED;
     const int nch = estimate_chunks(h, F, M, N, K * L);
     if (nch <= 1) {
+        if (pnce::mst_fuses(h, pilot)) {
+            pnce::TraceScope tr(h, s, pnce::TRACE_CORRELATE);
+            return from_cuda(pnce::launch_mst_rows(pilot, static_cast<const float2*>(Y_dev), N, A,
+                                                   pnce::lagmap_contiguous(K * L), dtype,
+                                                   static_cast<float2*>(H_dev), s));
+        }
         const pnce::QuantLayout lay = pnce::quant_layout(A, N, dtype);
         {
             pnce::TraceScope tr(h, s, pnce::TRACE_QUANTIZE);
@@ -430,6 +436,10 @@ pnce_status pnce_estimate_ex(pnce_handle* h, const pnce_pilot* pilot, const void
     const pnce::QuantLayout lay = pnce::quant_layout(A, N, dtype);
     if (workspace_bytes < lay.total) return PNCE_EINVAL;
     if (!(h->cc_major == 10 && h->cc_minor == 3)) return PNCE_EUNSUPPORTED;
+    if (pnce::mst_fuses(h, pilot)) {
+        pnce::TraceScope tr(h, s, pnce::TRACE_CORRELATE);
+        return from_cuda(pnce::launch_mst_rows(pilot, Y, stride, A, lm, dtype, H, s));
+    }
     {
         pnce::TraceScope tr(h, s, pnce::TRACE_QUANTIZE);
         st = from_cuda(pnce::launch_quantize(Y, A, N, dtype, pnce::ws_operand(workspace_dev, lay),
@@ -608,6 +618,10 @@ pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const vo
                 cst = from_cuda(pnce::launch_simt_bits(pilot, static_cast<const float2*>(yd), A,
                                                        N, K * L, static_cast<float2*>(hd),
                                                        h->s_comp));
+            } else if (pnce::mst_replaces_tc(pilot)) {
+                cst = from_cuda(pnce::launch_mst_rows(pilot, static_cast<const float2*>(yd), N, A,
+                                                      pnce::lagmap_contiguous(K * L), dtype,
+                                                      static_cast<float2*>(hd), h->s_comp));
             } else {
                 const pnce::QuantLayout ql = pnce::quant_layout(A, N, dtype);
                 void* q = ws + lay.q_off;

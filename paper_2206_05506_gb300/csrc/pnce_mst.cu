@@ -28,10 +28,14 @@
 // Against the dense sum (pnce_simt.cu): N = 4095, 2048 lags, 65536 rows 34.4 -> 0.67 ms;
 // N = 1023, 512 lags, 8192 rows 0.283 -> 0.028 ms; and closer to the 64-bit result (relative
 // error 0.7-1.0e-7 where the dense sum has 5e-7-1.1e-6: fewer roundings per output).
+#include <stdlib.h>
+
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "pnce_mst.h"
+#include "pnce_quant.h"
 
 namespace {
 
@@ -95,7 +99,28 @@ __device__ __forceinline__ void butterflies(float2 (&v)[E]) {
     }
 }
 
-template <int R, bool GRP>
+// v = round(v 2^s) in the format, s from the row's peak
+template <int DT, int E>
+__device__ __forceinline__ void round_entries(float2 (&v)[E], float sc) {
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+        v[k] = pnce::round_through<DT>(make_float2(v[k].x * sc, v[k].y * sc));
+}
+
+// The reduced formats (fp16, bf16, e4m3, tf32) take the same kernel: ROUND rounds the samples in
+// registers to what the quantiser would store (each value is exact in FP32), so the step is
+// one pass over Y with no operand in memory, and the sums keep all FP32 bits that the tensor
+// cores truncate.  One pass against quantise + tensor-core correlation: 65536 rows of
+// N = 4095, 2048 lags, fp16 1.43 -> 0.88 ms, e4m3 (32768 rows) 0.485 -> 0.42 ms; 8192 rows of
+// N = 1023, 512 lags, tf32 60 -> 29 us; relative error of the sums at N = 4095, fp16,
+// 1.4e-6 -> 1e-7.  CODES reads an operand that the quantiser has stored (traced calls, the
+// separate correlation step): the same bits.
+//
+// What a row is: FP32 samples (PLAIN), FP32 samples to be rounded to a reduced format first
+// (ROUND), or codes that the quantiser has stored (CODES).
+enum { PLAIN = 0, ROUND = 1, CODES = 2 };
+
+template <int R, bool GRP, int MODE>
 __global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
 mst_kernel(const pnce::MstLaunch p) {
     using M = Mst<R>;
@@ -119,7 +144,8 @@ mst_kernel(const pnce::MstLaunch p) {
 
     // as a programmatic dependent the tables came in beside the kernel before; the row map
     // and the rows are read only after it has finished
-    if constexpr (GRP) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (GRP || MODE == CODES) asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ float s_peak[16][8];                // peaks of a team's warps
 
     const int team = tid / M::TEAM, t = tid % G, sub = (tid % M::TEAM) / G;
     float2* buf = reinterpret_cast<float2*>(mst_smem + M::TAB) + (team * M::RT + sub) * M::ROW;
@@ -150,7 +176,30 @@ mst_kernel(const pnce::MstLaunch p) {
         if constexpr (GRP) {                       // a team without a row has nothing to do
             if (M::RT == 1 ? y == nullptr : __all_sync(0xffffffffu, y == nullptr)) continue;
         }
-        if (y) {
+        if constexpr (MODE == CODES) {
+            if (row < p.A) {
+                const unsigned char* op = static_cast<const unsigned char*>(p.operand);
+                const unsigned char* re = op + pnce::operand_row(row, 0) * p.op_pitch;
+                const unsigned char* im = op + pnce::operand_row(row, 1) * p.op_pitch;
+#pragma unroll
+                for (int i8 = 0; i8 < E / 8; ++i8) {
+                    const uint4 q = in_slot[i8 * G + t];
+                    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+                    float2 x[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int n = t + G * (8 * i8 + e);
+                        x[e] = make_float2(0.f, 0.f);           // entry 0 of X is zero
+                        if (n < p.N)
+                            x[e] = make_float2(pnce::decode(p.dtype, re, n),
+                                               pnce::decode(p.dtype, im, n));
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        buf[(e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu] = x[e];
+                }
+            }
+        } else if (y) {
 #pragma unroll
             for (int i8 = 0; i8 < E / 8; ++i8) {
                 const uint4 q = in_slot[i8 * G + t];
@@ -164,7 +213,7 @@ mst_kernel(const pnce::MstLaunch p) {
                 }
             }
         }
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        if constexpr (MODE != CODES) asm volatile("cp.async.wait_all;\n" ::: "memory");
         team_sync<M::TEAM>(team);
 
         float2 v[E];
@@ -176,6 +225,36 @@ mst_kernel(const pnce::MstLaunch p) {
             for (int e = 0; e < 8; ++e) {
                 const int k = 8 * k8 + e;
                 v[k] = buf[k * G + (t & ~15) + ((c >> (4 * e)) & 15u)];
+            }
+        }
+        float scale = p.invN;
+        if constexpr (MODE == CODES) {
+            if (row < p.A) scale = __ldg(p.factors + row);
+        }
+        if constexpr (MODE == ROUND) {
+            int se = 0;
+            if (p.target != 0) {
+                float m = 0.f;                     // NaN parts are left out, as fmaxf does
+#pragma unroll
+                for (int k = 0; k < E; ++k) m = fmaxf(m, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
+#pragma unroll
+                for (int o = (G < 32 ? G : 32) / 2; o; o >>= 1)
+                    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if constexpr (G > 32) {
+                    if ((t & 31) == 0) s_peak[team][t >> 5] = m;
+                    team_sync<M::TEAM>(team);
+#pragma unroll
+                    for (int w = 0; w < G / 32; ++w) m = fmaxf(m, s_peak[team][w]);
+                }
+                se = pnce::scale_exponent(p.target, m);
+                scale = ldexpf(p.invN, -se);
+            }
+            const float sc = ldexpf(1.0f, se);
+            switch (p.dtype) {
+                case PNCE_FP16: round_entries<PNCE_FP16>(v, sc); break;
+                case PNCE_BF16: round_entries<PNCE_BF16>(v, sc); break;
+                case PNCE_TF32: round_entries<PNCE_TF32>(v, sc); break;
+                default: round_entries<PNCE_FP8E4M3>(v, sc); break;
             }
         }
         butterflies<E, 1, E>(v);
@@ -227,11 +306,21 @@ mst_kernel(const pnce::MstLaunch p) {
                     lag = k * p.lags.step + (c - k * p.lags.L);
                 }
                 const float2 w = buf[lag_slot[lag]];
-                h[c] = make_float2(w.x * p.invN, w.y * p.invN);
+                h[c] = make_float2(w.x * scale, w.y * scale);
             }
         }
         team_sync<M::TEAM>(team);                  // the buffer takes the next row
     }
+}
+
+using MstKernel = void (*)(const pnce::MstLaunch);
+
+template <int R>
+MstKernel kernel_of(bool grp, int mode) {
+    if (grp) return mode == ROUND ? mst_kernel<R, true, ROUND> : mst_kernel<R, true, PLAIN>;
+    return mode == PLAIN   ? mst_kernel<R, false, PLAIN>
+           : mode == ROUND ? mst_kernel<R, false, ROUND>
+                           : mst_kernel<R, false, CODES>;
 }
 
 template <int R>
@@ -240,37 +329,26 @@ cudaError_t launch_r(const pnce::MstTables& m, const pnce::MstLaunch& p, cudaStr
     // rows spread over the SMs first, then over the teams of a block
     const long long teams = (p.A + M::RT - 1) / M::RT;
     const long long sms = m.num_sms;
-    const int max_teams = m.block_teams;
     long long per = (teams + sms - 1) / sms;
-    if (per > max_teams) per = max_teams;
+    if (per > m.block_teams) per = m.block_teams;
     long long grid = (teams + per - 1) / per;
-    const long long resident = sms * (per == max_teams ? m.blocks_per_sm : 1);
+    const long long resident = sms * (per == m.block_teams ? m.blocks_per_sm : 1);
     if (grid > resident) grid = resident;
-    const size_t smem = M::TAB + (size_t)per * M::team_bytes();
-    const unsigned block = (unsigned)(per * M::TEAM);
-    const bool grp = p.dd != nullptr;
-    if (p.pdl) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)grid, 1, 1);
-        cfg.blockDim = dim3(block, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        return grp ? cudaLaunchKernelEx(&cfg, mst_kernel<R, true>, p)
-                   : cudaLaunchKernelEx(&cfg, mst_kernel<R, false>, p);
-    }
-    if (grp)
-        mst_kernel<R, true><<<(unsigned)grid, block, smem, s>>>(p);
-    else
-        mst_kernel<R, false><<<(unsigned)grid, block, smem, s>>>(p);
-    return cudaGetLastError();
+    const int mode = p.operand ? CODES : p.dtype != PNCE_FP32_SIMT ? ROUND : PLAIN;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)(per * M::TEAM), 1, 1);
+    cfg.dynamicSmemBytes = M::TAB + (size_t)per * M::team_bytes();
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = p.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel_of<R>(p.dd != nullptr, mode), p);
 }
 
-// Shared-memory limits of both kernels, and how many teams fit an SM.
+// Shared-memory limits of the kernels, and how many teams fit an SM.
 template <int R>
 cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
     using M = Mst<R>;
@@ -280,15 +358,16 @@ cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
     if (teams > fit) teams = fit;
     const int smem = M::TAB + teams * (int)M::team_bytes();
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(mst_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  smem)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(mst_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  smem)) != cudaSuccess)
-        return e;
+    for (const auto& km : {std::make_pair(false, (int)PLAIN), std::make_pair(false, (int)ROUND),
+                           std::make_pair(false, (int)CODES), std::make_pair(true, (int)PLAIN),
+                           std::make_pair(true, (int)ROUND)})
+        if ((e = cudaFuncSetAttribute(kernel_of<R>(km.first, km.second),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
+            cudaSuccess)
+            return e;
     m.block_teams = teams;
     int per = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mst_kernel<R, false>,
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of<R>(false, PLAIN),
                                                            teams * M::TEAM, smem)) != cudaSuccess)
         return e;
     m.blocks_per_sm = per < 1 ? 1 : per;
@@ -415,8 +494,21 @@ cudaError_t mst_setup(MstTables& m, const uint16_t* tab_dev, int N, int num_sms,
     return e;
 }
 
+bool mst_replaces_tc(const pnce_pilot* pilot) {
+    if (!pilot->mst.tab) return false;
+    for (const char* name : {"PNCE_TC_PAIRS", "PNCE_TC_STAGED_PILOT", "PNCE_TC_LAGMAJOR",
+                             "PNCE_TC_LAGMAJOR_CL", "PNCE_TC_SMALL_GRID_BN",
+                             "PNCE_TC_TEST_DROP_ARRIVE", "PNCE_TC_FORCE"})
+        if (getenv(name)) return false;
+    return true;
+}
+
 cudaError_t launch_mst(const MstTables& m, MstLaunch p, cudaStream_t s) {
     if (p.A <= 0) return cudaSuccess;
+    p.target = p.dtype == PNCE_FP16      ? Fmt<PNCE_FP16>::target
+               : p.dtype == PNCE_FP8E4M3 ? Fmt<PNCE_FP8E4M3>::target
+                                         : 0;
+    p.op_pitch = (long long)row_pitch(m.N) * elem_bytes(p.dtype);
     p.tab = m.tab;
     p.N = m.N;
     p.invN = (float)(1.0 / (double)m.N);

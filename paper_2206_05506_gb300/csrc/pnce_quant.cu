@@ -8,38 +8,18 @@
 // writes rows operand_row(a, 0) (real) and operand_row(a, 1) (imaginary) of
 // round(y 2^s_a), four samples per thread per step.  Blocks past the last antenna zero
 // the padding rows of the last 8-antenna group.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include "pnce_internal.h"
+#include "pnce_quant.h"
 
 namespace {
 
+using pnce::Fmt;
+using pnce::to_bf16;
+using pnce::to_e4m3x2;
+using pnce::to_f16;
+using pnce::to_tf32;
+
 constexpr int THREADS = 256;
-
-template <int DT> struct Fmt;
-template <> struct Fmt<PNCE_FP16> { static constexpr int target = 15; using T = uint16_t; };
-template <> struct Fmt<PNCE_BF16> { static constexpr int target = 0; using T = uint16_t; };
-template <> struct Fmt<PNCE_TF32> { static constexpr int target = 0; using T = uint32_t; };
-template <> struct Fmt<PNCE_FP8E4M3> { static constexpr int target = 8; using T = uint8_t; };
-
-__device__ __forceinline__ uint16_t to_f16(float x) {
-    return __half_as_ushort(__float2half_rn(x));
-}
-__device__ __forceinline__ uint16_t to_bf16(float x) {
-    return __bfloat16_as_ushort(__float2bfloat16_rn(x));
-}
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
-// two e4m3 codes (lo from a, hi from b), round to nearest even, saturate to +-448
-__device__ __forceinline__ uint16_t to_e4m3x2(float a, float b) {
-    uint16_t r;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %2, %1;" : "=h"(r) : "f"(a), "f"(b));
-    return r;
-}
 
 // write four consecutive converted values v[0..3] at element n of row `row`
 template <int DT>
@@ -129,13 +109,7 @@ quantize_kernel(const float2* __restrict__ Y, long long A, int N, long long y_st
             m = fmaxf(m, s_max[w]);
             et += s_pow[w];
         }
-        int se = 0;
-        if (Fmt<DT>::target != 0 && m > 0.f && isfinite(m)) {
-            int ex;
-            frexpf(m, &ex);                          // m = mant * 2^ex, mant in [0.5, 1)
-            se = Fmt<DT>::target - ex;
-            se = se < -100 ? -100 : (se > 100 ? 100 : se);
-        }
+        const int se = pnce::scale_exponent(Fmt<DT>::target, m);
         s_scale = ldexpf(1.0f, se);
         out_scale[a] = ldexpf(invN, -se);
         if (exps) exps[a] = se;
@@ -255,13 +229,7 @@ grouped_quantize_kernel(const pnce_req_desc* __restrict__ dd, const int* __restr
     if (tid == 0) {
         float m = 0.f;
         for (int w = 0; w < THREADS / 32; ++w) m = fmaxf(m, s_max[w]);
-        int se = 0;
-        if (Fmt<DT>::target != 0 && m > 0.f && isfinite(m)) {
-            int ex;
-            frexpf(m, &ex);
-            se = Fmt<DT>::target - ex;
-            se = se < -100 ? -100 : (se > 100 ? 100 : se);
-        }
+        const int se = pnce::scale_exponent(Fmt<DT>::target, m);
         s_scale = ldexpf(1.0f, se);
         out_scale[a] = ldexpf(invN, -se);
     }

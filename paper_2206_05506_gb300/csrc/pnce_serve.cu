@@ -236,23 +236,27 @@ pnce_status pnce_estimate_grouped(pnce_handle* h, const pnce_pilot* pilot,
     pnce_req_desc* dd = reinterpret_cast<pnce_req_desc*>(ws + lay.d_off);
     int* row_req = reinterpret_cast<int*>(ws + lay.m_off);
     // prep (table copy + row map), then every kernel as a programmatic dependent of the one
-    // before it: four graph nodes on the tensor-core path (prep, gather-quantise,
-    // correlation, scatter), two or three on the FP32 path (prep, a row gather when the lags
-    // span several tiles, the correlation writing into the requests' results)
+    // before it: with an m-sequence pilot the transform, reading from and writing into the
+    // requests' buffers (two graph nodes); with other pilots four nodes on the tensor-core path
+    // (prep, gather-quantise, correlation, scatter), two or three on the FP32 path (prep, a
+    // row gather when the lags span several tiles, the correlation writing into the requests'
+    // results)
     grouped_prep_kernel<<<1, PREP_THREADS, 0, s>>>(descs, nreq, rows, kl_max, dd, row_req,
                                                    h->status_dev);
     if (cudaGetLastError() != cudaSuccess) return PNCE_ECUDA;
+    if (dtype == PNCE_FP32_SIMT ? pilot->mst.tab != nullptr : pnce::mst_fuses(h, pilot)) {
+        pnce::MstLaunch l;
+        l.A = rows;
+        l.lags = pnce::lagmap_contiguous(kl_max);
+        l.dd = dd;
+        l.row_req = row_req;
+        l.pdl = !h->trace_on;
+        l.dtype = dtype;
+        pnce::TraceScope tr(h, s, dtype == PNCE_FP32_SIMT ? pnce::TRACE_SIMT
+                                                          : pnce::TRACE_CORRELATE);
+        return pnce::launch_mst(pilot->mst, l, s) == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
+    }
     if (dtype == PNCE_FP32_SIMT) {
-        if (pilot->mst.tab) {
-            pnce::MstLaunch l;
-            l.A = rows;
-            l.lags = pnce::lagmap_contiguous(kl_max);
-            l.dd = dd;
-            l.row_req = row_req;
-            l.pdl = !h->trace_on;
-            pnce::TraceScope tr(h, s, pnce::TRACE_SIMT);
-            return pnce::launch_mst(pilot->mst, l, s) == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
-        }
         float2* Yb = reinterpret_cast<float2*>(ws + lay.y_off);
         if (pnce::simt_grouped_ok(N, kl_max)) {
             // the SIMT kernel writes each row's lags into its request; it reads the rows

@@ -674,15 +674,8 @@ cudaError_t launch_simt_grouped(const pnce_pilot* pilot, const pnce_req_desc* dd
 cudaError_t launch_simt_bits_ex(const pnce_pilot* pilot, const float2* Y, long long y_stride,
                                 long long A, int N, const LagMap& lags, float2* H,
                                 cudaStream_t s) {
-    if (pilot->mst.tab && !(lags.mode == 0 && lags.ldH <= FEW_LAGS)) {
-        MstLaunch l;
-        l.Y = Y;
-        l.y_stride = y_stride;
-        l.A = A;
-        l.lags = lags;
-        l.H = H;
-        return launch_mst(pilot->mst, l, s);
-    }
+    if (pilot->mst.tab && !(lags.mode == 0 && lags.ldH <= FEW_LAGS))
+        return launch_mst_rows(pilot, Y, y_stride, A, lags, PNCE_FP32_SIMT, H, s);
     if (lags.mode == 0 && lags.ldH <= FEW_LAGS)
         return launch_few_lags(pilot->ext_bits_dev, Y, y_stride, A, N, lags.ldH, lags.ldH, H, s);
     return launch<FWD_BITS>(pilot->ext_bits_dev, nullptr, Y, y_stride, A, N, lags, N, H, s);

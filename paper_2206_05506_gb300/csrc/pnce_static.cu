@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -54,12 +55,18 @@ extern "C" pnce_status pnce_estimate_static(pnce_handle* h, const pnce_pilot* pi
     if (dev != h->device || pilot->device != h->device) return PNCE_ESTATE;
     if (pilot->N != N) return PNCE_ESTATE;
     if (!(h->cc_major == 10 && h->cc_minor == 3)) return PNCE_EUNSUPPORTED;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (pnce::mst_fuses(h, pilot))       // one launch that rounds in registers: no scratch
+        return pnce::launch_mst_rows(pilot, static_cast<const float2*>(Y_dev), N, A,
+                                     pnce::lagmap_contiguous(K * L), dtype,
+                                     static_cast<float2*>(H_dev), s) == cudaSuccess
+                   ? PNCE_OK
+                   : PNCE_ECUDA;
     void* ws = nullptr;
     pnce_status st = scratch_address(dev, &ws);
     if (st != PNCE_OK) return st;
     // nothing in the scratch needs clearing: every row and factor the correlation reads is
     // rewritten by the quantiser first, and the pad columns past N are never read
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     const pnce::QuantLayout lay = pnce::quant_layout(A, N, dtype);
     {
         pnce::TraceScope tr(h, s, pnce::TRACE_QUANTIZE);

@@ -43,6 +43,7 @@
 #include <mutex>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -1814,6 +1815,17 @@ pnce_status launch_tc_ex(const pnce_handle* h, const pnce_pilot* pilot, long lon
                          const LagMap& lm, int dtype, const void* operand, const float* factors,
                          float2* H, cudaStream_t s, bool pdl) {
     if (!(h->cc_major == 10 && h->cc_minor == 3)) return PNCE_EUNSUPPORTED;
+    if (mst_replaces_tc(pilot)) {
+        MstLaunch l;
+        l.A = A;
+        l.lags = lm;
+        l.H = H;
+        l.pdl = pdl;
+        l.dtype = dtype;
+        l.operand = operand;
+        l.factors = factors;
+        return launch_mst(pilot->mst, l, s) == cudaSuccess ? PNCE_OK : PNCE_ECUDA;
+    }
     switch (dtype) {
         case PNCE_FP16:
             return launch_dt<PNCE_FP16>(h, pilot, A, N, lm, operand, factors, H, s, pdl);

@@ -101,3 +101,69 @@ def test_other_bits_keep_the_dense_kernel():
     Y = _y(np.random.default_rng(3), 2, 9, bits.size)
     H = pk.estimate(torch.from_numpy(Y).to(dev), pk.Pilot(bits, device=dev), 2, 64, dtype="fp32")
     assert O.nmse(H.cpu().numpy(), O.estimate(Y, bits, 2, 64)) <= TOL
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16", "e4m3", "tf32"])
+@pytest.mark.parametrize("r", range(7, 15))
+def test_reduced_formats_in_one_launch(r, dtype, monkeypatch):
+    # rounding in registers gives the bits that quantise-then-correlate gives, both are the
+    # FP64 estimate of the quantised operand, and the tensor cores agree to their accumulation;
+    # powers over decades, zero rows, samples that are not numbers
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 2)
+    N, A, K, L = bits.size, 11, 3, 19
+    rng = np.random.default_rng([r, 5])
+    Y = _y(rng, 1, A, N) * np.logspace(-4, 4, A, dtype=np.float32)[None, :, None]
+    Y[0, 4] = 0
+    pilot = pk.Pilot(bits, device=dev)
+    Yd = torch.from_numpy(Y).to(dev)
+    H = pk.estimate(Yd, pilot, K, L, dtype=dtype)
+    q = pk.quantize(Yd, dtype)
+    assert torch.equal(pk.correlate_quantized(q["workspace"], pilot, 1, A, K, L, dtype), H)
+    ref = O.estimate_quantized(Y, bits, K, L, dtype)
+    assert O.nmse(H.cpu().numpy(), ref) <= TOL
+    Ys = torch.cat([torch.zeros(1, A, 4, dtype=torch.complex64, device=dev), Yd], dim=2)
+    Hs = pk.estimate(Ys, pilot, K, L, dtype=dtype, cp_len=4, shift_rule="spread")
+    odd = Yd.clone()
+    odd[0, 0, 3], odd[0, 1, 7], odd[0, 2, N - 1] = complex(float("nan"), 1), complex(0, float("inf")), complex(float("-inf"), 2)
+    Ho = pk.estimate(odd, pilot, K, L, dtype=dtype)
+    monkeypatch.setenv("PNCE_TC_FORCE", "1")                 # the tensor-core kernels
+    Ht = pk.estimate(Yd, pilot, K, L, dtype=dtype)
+    assert O.nmse(Ht.cpu().numpy(), ref) <= 1e-9
+    assert O.nmse(Hs.cpu().numpy(), pk.estimate(Ys, pilot, K, L, dtype=dtype, cp_len=4,
+                                                shift_rule="spread").cpu().numpy()) <= 1e-9
+    Hto = torch.view_as_real(pk.estimate(odd, pilot, K, L, dtype=dtype))
+    Ho = torch.view_as_real(Ho)
+    assert torch.equal(torch.isnan(Ho), torch.isnan(Hto))
+    assert torch.equal(torch.isinf(Ho), torch.isinf(Hto))
+    assert torch.equal(torch.sign(Ho[torch.isinf(Ho)]), torch.sign(Hto[torch.isinf(Hto)]))
+    assert pk.get_status(dev) == 0
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16", "e4m3", "tf32"])
+def test_other_bits_keep_the_tensor_cores(dtype):
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    for r, F, M, K, L in [(7, 1, 8, 2, 16), (10, 3, 100, 5, 60), (12, 2, 64, 16, 128)]:
+        bits = mseq.mseq_bits(r, 0).copy()
+        bits[5] ^= 1
+        Y = _y(np.random.default_rng(r), F, M, bits.size)
+        H = pk.estimate(torch.from_numpy(Y).to(dev), pk.Pilot(bits, device=dev), K, L, dtype=dtype)
+        assert O.nmse(H.cpu().numpy(), O.estimate_quantized(Y, bits, K, L, dtype)) <= 1e-9
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "fp16", "e4m3"])
+def test_traced_calls_give_the_same_bits(dtype):
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(11, 0)
+    pilot = pk.Pilot(bits, device=dev)
+    Y = torch.from_numpy(_y(np.random.default_rng(1), 2, 21, bits.size)).to(dev)
+    H = pk.estimate(Y, pilot, 4, 50, dtype=dtype)
+    pk.trace_enable(True, dev)
+    Ht = pk.estimate(Y, pilot, 4, 50, dtype=dtype)
+    kinds = [k for k, _ in pk.trace_read(dev)]
+    pk.trace_enable(False, dev)
+    assert torch.equal(H, Ht)
+    assert kinds == (["simt"] if dtype == "fp32" else ["quantize", "correlate"])
