@@ -1,4 +1,5 @@
-// Adjoint of the real-pilot correlation (pilot optimisation through the estimator).
+// Adjoint of the real-pilot correlation (pilot optimisation through the estimator): the
+// entry to it, and the dense kernels for shapes beyond the transform lengths of pnce_fft.cu.
 //
 // Forward: H[a][j] = (1/N) sum_n Y[a][n] p[(n - j) mod N], p real.  For a real loss with
 // G = dLoss/dRe(H) + i dLoss/dIm(H):
@@ -232,7 +233,7 @@ cudaError_t launch_dp(const DpGrid& g, const float2* G, const float2* Y, long lo
 namespace pnce {
 
 size_t backward_workspace(long long A, int N, int KL) {
-    (void)KL;
+    if (fft_applies(N, KL)) return fft_adjoint_workspace(A, N, KL);
     const DpGrid g = dp_grid(A, N);
     return round_up((size_t)(g.P * g.Q) * (size_t)g.QT * sizeof(float), 256);
 }
@@ -240,12 +241,13 @@ size_t backward_workspace(long long A, int N, int KL) {
 cudaError_t launch_backward(const float* p, bool tanh_map, const float2* Y, const float2* G,
                             long long A, int N, int KL, float2* dY, float* dp, void* ws,
                             size_t ws_bytes, cudaStream_t s) {
+    if (dp && ws_bytes < backward_workspace(A, N, KL)) return cudaErrorInvalidValue;
+    if (fft_applies(N, KL)) return launch_fft_adjoint(p, tanh_map, G, Y, A, N, KL, dY, dp, ws, s);
     if (dY) {
         cudaError_t e = launch_adjoint_dy(p, tanh_map, G, A, N, KL, dY, s);
         if (e != cudaSuccess) return e;
     }
     if (dp) {
-        if (ws_bytes < backward_workspace(A, N, KL)) return cudaErrorInvalidValue;
         const DpGrid g = dp_grid(A, N);
         float* partial = static_cast<float*>(ws);
         cudaError_t e = g.R == 8 ? launch_dp<8>(g, G, Y, A, N, KL, partial, s)

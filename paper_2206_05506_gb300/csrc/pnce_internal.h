@@ -215,6 +215,16 @@ cudaError_t launch_backward(const float* p, bool tanh_map, const float2* Y, cons
 cudaError_t launch_adjoint_dy(const float* p, bool tanh_map, const float2* G, long long A, int N,
                               int KL, float2* dY, cudaStream_t s);
 size_t backward_workspace(long long A, int N, int KL);
+// Real-valued pilots by FFT (pnce_fft.cu), for shapes whose transform length is at most 4096:
+// forward, and the adjoint (dY and dp either may be null; ws: fft_adjoint_workspace bytes, for
+// dp only).
+bool fft_applies(int N, int KL);
+cudaError_t launch_fft_forward(const float* p, bool tanh_map, const float2* Y, long long A, int N,
+                               int KL, float2* H, cudaStream_t s);
+size_t fft_adjoint_workspace(long long A, int N, int KL);
+cudaError_t launch_fft_adjoint(const float* p, bool tanh_map, const float2* G, const float2* Y,
+                               long long A, int N, int KL, float2* dY, float* dp, void* ws,
+                               cudaStream_t s);
 // copy `bytes` (a multiple of 8) from device memory into page-locked host memory with a
 // kernel of at most num_sms blocks; dst must be the device-visible address of the
 // page-locked buffer

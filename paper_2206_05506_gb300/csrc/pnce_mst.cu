@@ -161,7 +161,7 @@ mst_kernel(const pnce::MstLaunch p) {
         int cols = p.lags.ldH;
         if (row < p.A) {
             if constexpr (GRP) {
-                const int b = __ldg(p.row_req + row);
+                const int b = p.row_req[row];     // a plain load: it stays behind the wait
                 if (b >= 0) {
                     const pnce_req_desc& q = p.dd[b];
                     cols = q.K * q.L;
@@ -229,7 +229,7 @@ mst_kernel(const pnce::MstLaunch p) {
         }
         float scale = p.invN;
         if constexpr (MODE == CODES) {
-            if (row < p.A) scale = __ldg(p.factors + row);
+            if (row < p.A) scale = p.factors[row];
         }
         if constexpr (MODE == ROUND) {
             int se = 0;
