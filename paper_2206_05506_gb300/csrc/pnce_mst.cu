@@ -21,11 +21,14 @@
 //    is found by four halvings of the graph.  The same on the way out.  Addressed by s itself,
 //    the scatter and the gather each took about 3 wavefronts for every one they need.
 //    (With the r <= 8 levels of a pass done by lane shuffles and X addressed by s, 512 frames x
-//    128 rows of N = 4095 with 2048 lags took 0.93 ms; now 0.67 ms, 4.8 TB/s.)
+//    128 rows of N = 4095 with 2048 lags took 0.93 ms; without, 0.67 ms.)
 //  * A team of G = 2^r / E threads (one warp or less for r <= 11) owns a row; teams only
 //    synchronise within themselves, so the rows of an SM sit in different phases and the
-//    loads of some overlap the additions of others.
-// Against the dense sum (pnce_simt.cu): N = 4095, 2048 lags, 65536 rows 34.4 -> 0.67 ms;
+//    loads of some overlap the additions of others.  The registers and the buffer of a team
+//    hold one row only, so it asks L2 for its next row while it works on this one: its load
+//    phase then waits for L2, not for memory.  65536 rows of N = 4095, 2048 lags: 0.68 -> 0.56
+//    ms (5.7 TB/s); 131072 rows of N = 1023, 512 lags: 277 -> 248 us (6.5 TB/s, 0.95 of a copy).
+// Against the dense sum (pnce_simt.cu): N = 4095, 2048 lags, 65536 rows 34.4 -> 0.56 ms;
 // N = 1023, 512 lags, 8192 rows 0.283 -> 0.028 ms; and closer to the 64-bit result (relative
 // error 0.7-1.0e-7 where the dense sum has 5e-7-1.1e-6: fewer roundings per output).
 #include <stdlib.h>
@@ -83,6 +86,13 @@ __device__ __forceinline__ void cp_async8(unsigned smem, const void* gmem, int b
                  : "memory");
 }
 
+// asks for the 16-byte units that lie within n samples
+__device__ __forceinline__ void prefetch_l2(const float2* row, int n) {
+    const uintptr_t a = ((uintptr_t)row + 15) & ~(uintptr_t)15;
+    const unsigned bytes = (unsigned)((uintptr_t)(row + n) - a) & ~15u;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
+}
+
 // butterfly levels on register distances FIRST, 2 FIRST, .. < LAST
 template <int E, int FIRST, int LAST>
 __device__ __forceinline__ void butterflies(float2 (&v)[E]) {
@@ -111,8 +121,8 @@ __device__ __forceinline__ void round_entries(float2 (&v)[E], float sc) {
 // registers to what the quantiser would store (each value is exact in FP32), so the step is
 // one pass over Y with no operand in memory, and the sums keep all FP32 bits that the tensor
 // cores truncate.  One pass against quantise + tensor-core correlation: 65536 rows of
-// N = 4095, 2048 lags, fp16 1.43 -> 0.88 ms, e4m3 (32768 rows) 0.485 -> 0.42 ms; 8192 rows of
-// N = 1023, 512 lags, tf32 60 -> 29 us; relative error of the sums at N = 4095, fp16,
+// N = 4095, 2048 lags, fp16 1.43 -> 0.78 ms, e4m3 (32768 rows) 0.485 -> 0.347 ms; 8192 rows of
+// N = 1023, 512 lags, tf32 60 -> 27 us; relative error of the sums at N = 4095, fp16,
 // 1.4e-6 -> 1e-7.  CODES reads an operand that the quantiser has stored (traced calls, the
 // separate correlation step): the same bits.
 //
@@ -214,6 +224,9 @@ mst_kernel(const pnce::MstLaunch p) {
             }
         }
         if constexpr (MODE != CODES) asm volatile("cp.async.wait_all;\n" ::: "memory");
+        if constexpr (!GRP && MODE != CODES) {
+            if (t == 0 && row + stride < p.A) prefetch_l2(y + stride * p.y_stride, p.N);
+        }
         team_sync<M::TEAM>(team);
 
         float2 v[E];
