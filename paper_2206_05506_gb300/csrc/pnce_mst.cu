@@ -117,11 +117,31 @@ __device__ __forceinline__ void round_entries(float2 (&v)[E], float sc) {
         v[k] = pnce::round_through<DT>(make_float2(v[k].x * sc, v[k].y * sc));
 }
 
+// The same for fp16 and e4m3 where no |v 2^s| rounds above the format's largest number, in
+// FP32 arithmetic: adding and taking away 1.5 x 2^(e + D), e the exponent of v 2^s but not less
+// than the format's smallest, leaves v 2^s rounded to even at the format's last place (a NaN
+// stays one).  Conversions to and from the formats seem to issue at 16 a clock per SM and held
+// the kernel up: 65536 rows of N = 4095, 2048 lags, fp16 0.78 -> 0.65 ms; e4m3, 32768 rows, 0.347
+// -> 0.337 ms.  (bf16 and tf32 need one and two conversions per sample: 0.33 ms both.)
+template <int DT, int E>
+__device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
+    constexpr int D = DT == PNCE_FP16 ? 13 : 20, EMIN = DT == PNCE_FP16 ? -14 : -6;
+    const int add = (D + se) * (1 << 23) + 0x400000, least = (127 + EMIN + D) * (1 << 23) + 0x400000;
+    const float2 sc2 = make_float2(sc, sc), m1 = make_float2(-1.f, -1.f);
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        const float2 big = make_float2(
+            __int_as_float(max((__float_as_int(v[k].x) & 0x7f800000) + add, least)),
+            __int_as_float(max((__float_as_int(v[k].y) & 0x7f800000) + add, least)));
+        v[k] = __ffma2_rn(big, m1, __ffma2_rn(v[k], sc2, big));
+    }
+}
+
 // The reduced formats (fp16, bf16, e4m3, tf32) take the same kernel: ROUND rounds the samples in
 // registers to what the quantiser would store (each value is exact in FP32), so the step is
 // one pass over Y with no operand in memory, and the sums keep all FP32 bits that the tensor
 // cores truncate.  One pass against quantise + tensor-core correlation: 65536 rows of
-// N = 4095, 2048 lags, fp16 1.43 -> 0.78 ms, e4m3 (32768 rows) 0.485 -> 0.347 ms; 8192 rows of
+// N = 4095, 2048 lags, fp16 1.43 -> 0.65 ms, e4m3 (32768 rows) 0.485 -> 0.337 ms; 8192 rows of
 // N = 1023, 512 lags, tf32 60 -> 27 us; relative error of the sums at N = 4095, fp16,
 // 1.4e-6 -> 1e-7.  CODES reads an operand that the quantiser has stored (traced calls, the
 // separate correlation step): the same bits.
@@ -246,8 +266,8 @@ mst_kernel(const pnce::MstLaunch p) {
         }
         if constexpr (MODE == ROUND) {
             int se = 0;
-            if (p.target != 0) {
-                float m = 0.f;                     // NaN parts are left out, as fmaxf does
+            float m = 0.f;
+            if (p.target != 0) {                   // NaN parts are left out, as fmaxf does
 #pragma unroll
                 for (int k = 0; k < E; ++k) m = fmaxf(m, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
 #pragma unroll
@@ -263,11 +283,18 @@ mst_kernel(const pnce::MstLaunch p) {
                 scale = ldexpf(p.invN, -se);
             }
             const float sc = ldexpf(1.0f, se);
-            switch (p.dtype) {
-                case PNCE_FP16: round_entries<PNCE_FP16>(v, sc); break;
-                case PNCE_BF16: round_entries<PNCE_BF16>(v, sc); break;
-                case PNCE_TF32: round_entries<PNCE_TF32>(v, sc); break;
-                default: round_entries<PNCE_FP8E4M3>(v, sc); break;
+            const bool small = m * sc < ldexpf(1.0f, p.target);   // no code overflows
+            if (p.dtype == PNCE_FP16 && small) {
+                round_small<PNCE_FP16>(v, sc, se);
+            } else if (p.dtype == PNCE_FP8E4M3 && small) {
+                round_small<PNCE_FP8E4M3>(v, sc, se);
+            } else {
+                switch (p.dtype) {
+                    case PNCE_FP16: round_entries<PNCE_FP16>(v, sc); break;
+                    case PNCE_BF16: round_entries<PNCE_BF16>(v, sc); break;
+                    case PNCE_TF32: round_entries<PNCE_TF32>(v, sc); break;
+                    default: round_entries<PNCE_FP8E4M3>(v, sc); break;
+                }
             }
         }
         butterflies<E, 1, E>(v);
