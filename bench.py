@@ -609,7 +609,7 @@ def run_layouts(dev, pilot, Y, K, L, taps_per_step, reps: int = 30):
 
 def run_small_case(dev, ref=None, calls: int = 200):
     """Launch-latency case: one frame of 8 antennas, N = 127, K = 2, L = 16 (8 KB in, 2 KB
-    out), FP32 (the few-lags SIMT kernel).  Per call: the kernel's device time (the
+    out), FP32 (the transform's few-lags form).  Per call: the kernel's device time (the
     library's trace events around the launch), the host wall time of the call and its
     synchronisation, and end to end from page-locked host memory (pnce_estimate_host: copy
     in, estimate, copy out).  ref: the oracle's result (from oracle_references) or None."""

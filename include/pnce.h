@@ -74,7 +74,9 @@ typedef enum {
  * PNCE_FP16 (the paper's tensor-core operand format, Sec. III-B).  With few lags the
  * correlation is bound by reading Y once (8 bytes per sample), which the FP32 kernel does
  * at about the rate of the quantiser pass that every tensor-core estimate starts with, so
- * exact FP32 costs nothing there; with more lags the tensor cores win by far.  Host only;
+ * exact FP32 costs nothing there; with more lags the tensor cores win by far, unless the
+ * pilot is an m-sequence with a fast transform (N = 127 .. 16383), where every dtype reads Y
+ * once.  Host only;
  * returns -1 for an invalid shape.  pnce_workspace_size, pnce_estimate, pnce_estimate_ex,
  * pnce_host_workspace_size, pnce_estimate_host, pnce_grouped_workspace_size and
  * pnce_estimate_grouped (with K*L = kl_max) accept PNCE_AUTO and resolve it by this rule;

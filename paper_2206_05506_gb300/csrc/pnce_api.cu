@@ -262,12 +262,13 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
     // the next 16-byte boundary on
     const size_t bits_bytes = pnce::round_up(sizeof(uint32_t) * (size_t)words, 16);
     size_t mst_bytes = pnce::mst_table_bytes(N);
+    size_t lag_bytes = mst_bytes ? sizeof(uint16_t) * ((size_t)N + 1) : 0;     // u_j after them
     std::vector<uint32_t> ext;
     try {
-        ext.assign((bits_bytes + mst_bytes) / sizeof(uint32_t), 0u);
-        if (mst_bytes &&
-            !pnce::mst_build_tables(bits_host, N, reinterpret_cast<uint16_t*>(ext.data() + bits_bytes / 4)))
-            mst_bytes = 0;
+        ext.assign((bits_bytes + mst_bytes + lag_bytes) / sizeof(uint32_t), 0u);
+        uint16_t* tab = reinterpret_cast<uint16_t*>(ext.data() + bits_bytes / 4);
+        if (mst_bytes && !pnce::mst_build_tables(bits_host, N, tab, tab + mst_bytes / 2))
+            mst_bytes = lag_bytes = 0;
     } catch (...) {
         return PNCE_ENOMEM;
     }
@@ -281,7 +282,7 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
     p->device = h->device;
     p->N = N;
     p->ext_words = words;
-    const size_t bytes = bits_bytes + mst_bytes;
+    const size_t bytes = bits_bytes + mst_bytes + lag_bytes;
     if (cudaMalloc(&p->ext_bits_dev, bytes) != cudaSuccess) {
         delete p;
         return PNCE_ENOMEM;
@@ -293,6 +294,7 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
         delete p;
         return PNCE_ECUDA;
     }
+    if (mst_bytes) p->mst.lagvec = tab + mst_bytes / 2;
     *out = p;
     return PNCE_OK;
 }

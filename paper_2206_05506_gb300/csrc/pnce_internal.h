@@ -89,6 +89,7 @@ namespace pnce {
 // pilot is no m-sequence of a supported degree) and the launch shape that fits an SM.
 struct MstTables {
     const uint16_t* tab = nullptr;
+    const uint16_t* lagvec = nullptr;   // vectors u_j of the lags, for few lags (may be null)
     int N = 0, r = 0;
     int num_sms = 0, block_teams = 0, blocks_per_sm = 0;
 };

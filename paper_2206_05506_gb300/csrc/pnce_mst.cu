@@ -33,6 +33,7 @@
 // error 0.7-1.0e-7 where the dense sum has 5e-7-1.1e-6: fewer roundings per output).
 #include <stdlib.h>
 
+#include <algorithm>
 #include <new>
 #include <utility>
 #include <vector>
@@ -60,6 +61,7 @@ struct Mst {
     // tables in shared memory; for r >= 13 they are read from global memory
     static constexpr bool TAB_SMEM = R <= 12;
     static constexpr int TAB = TAB_SMEM ? S * 6 + S / 2 : 0;
+    static constexpr int TAB_FEW = TAB_SMEM ? S * 2 + S / 2 : 0;     // the few-lags kernel's
     // most threads per block and most blocks per SM (registers: 2 E + about 40 each)
     static constexpr int MAXT = R >= 14 ? 256 : R >= 11 ? 384 : R >= 9 ? 640 : 512;
     static constexpr int MINB = R >= 9 ? 1 : 2;
@@ -150,7 +152,67 @@ __device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
 // (ROUND), or codes that the quantiser has stored (CODES).
 enum { PLAIN = 0, ROUND = 1, CODES = 2 };
 
-template <int R, bool GRP, int MODE>
+// Few lags (FEW): the second pass and the exchange before it would form all 2^r sums for a
+// handful.  Instead the registers' sums V_t[k] of the wanted rows k (the upper bits of the
+// columns' vectors u_j: at most one row per column) are left in the buffer, and P threads per
+// column add its G = 2^r / E values with their signs.  Taken for up to few_cols columns, where it
+// is the faster one, in us, with / without (1.07 GB of samples each, whatever r):
+//   r    12: 16 columns 181 / 231, 32 211 / 231, 48 268 / 231
+//        11: 16 173 / 208, 32 201 / 208, 48 223 / 208     10: 16 178 / 189, 32 258 / 191
+//         9: 8 169 / 188, 16 204 / 198     8: 8 173 / 191, 16 235 / 200     7: 8 218 / 249
+// Against one bit test and one addition per sample and lag (pnce_simt.cu), same sizes: r = 12,
+// 16 lags 253 -> 181, 8 lags 182 -> 174; r = 10, 16 lags 298 -> 178; r = 7, 8 lags 546 -> 218;
+// relative error 5.8-8.9e-8 -> 4.6-7.9e-8.
+constexpr int few_cols(int r) { return r >= 11 ? 32 : r == 10 ? 16 : 8; }
+
+// G (a power of two) values of one column: sum over t of (-1)^<ul, t> V_t, the P = 2^lgP
+// threads of the column taking every P-th each; the same on all P lanes.  row: V_t at
+// (t + rot) mod G.
+template <int G>
+__device__ __forceinline__ float2 column_sum(const float2* row, int rot, unsigned ul, int part,
+                                             int lgP) {
+    const int n = G >> lgP;
+    float2 acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = make_float2(0.f, 0.f);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        // bit i: the sign of value part + P (i0 + i)
+        const unsigned x = ul >> lgP;
+        unsigned w = (__popc(ul & (unsigned)(part + (i0 << lgP))) & 1) ? 0xffffffffu : 0u;
+        w ^= (x & 1u ? 0xaaaaaaaau : 0u) ^ (x & 2u ? 0xccccccccu : 0u) ^ (x & 4u ? 0xf0f0f0f0u : 0u) ^
+             (x & 8u ? 0xff00ff00u : 0u) ^ (x & 16u ? 0xffff0000u : 0u);
+        const int m = n < 32 ? n : 32;
+        for (int i = 0; i < m; i += 8) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                if (e < m) {
+                    const float2 v = row[(part + ((i0 + i + e) << lgP) + rot) & (G - 1)];
+                    const float sg = __uint_as_float((w << (31 - e) & 0x80000000u) | 0x3f800000u);
+                    acc[e] = __ffma2_rn(v, make_float2(sg, sg), acc[e]);
+                }
+            }
+            w >>= 8;
+        }
+    }
+#pragma unroll
+    for (int d = 4; d; d >>= 1)
+#pragma unroll
+        for (int e = 0; e < d; ++e) acc[e] = __fadd2_rn(acc[e], acc[e + d]);
+    float2 s = acc[0];
+    for (int o = 1; o < (1 << lgP); o <<= 1)
+        s = __fadd2_rn(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o),
+                                      __shfl_xor_sync(0xffffffffu, s.y, o)));
+    return s;
+}
+
+// column k L + l holds lag k step + l
+__device__ __forceinline__ int lag_of(const pnce::MstLaunch& p, int c) {
+    if (p.lags.mode == 0) return c;
+    const int k = (int)__umulhi((unsigned)c << 4, p.magic_L);
+    return k * p.lags.step + (c - k * p.lags.L);
+}
+
+template <int R, bool GRP, int MODE, bool FEW>
 __global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
 mst_kernel(const pnce::MstLaunch p) {
     using M = Mst<R>;
@@ -161,16 +223,33 @@ mst_kernel(const pnce::MstLaunch p) {
     if constexpr (M::TAB_SMEM) {
         const uint4* src = reinterpret_cast<const uint4*>(p.tab);
         uint4* dst = reinterpret_cast<uint4*>(mst_smem);
-        for (int i = tid; i < M::TAB / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+        if constexpr (FEW) {
+            for (int i = tid; i < M::TAB_FEW / 16; i += blockDim.x)
+                dst[i] = __ldg(src + (i < S / 8 ? i : i + S / 4));
+        } else {
+            for (int i = tid; i < M::TAB / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+        }
         tab = reinterpret_cast<const uint16_t*>(mst_smem);
-        __syncthreads();
     } else {
         tab = p.tab;
     }
+    __shared__ uint16_t few_u[few_cols(R)];      // u_j of the columns
+    __shared__ unsigned few_rows[2];               // rows k that they need
+    if constexpr (FEW) {
+        if (tid < 2) few_rows[tid] = 0;
+        __syncthreads();
+        for (int c = tid; c < p.lags.ldH; c += blockDim.x) {
+            const unsigned u = __ldg(p.lagvec + lag_of(p, c));
+            few_u[c] = (uint16_t)u;
+            atomicOr(&few_rows[u >> LG >> 5], 1u << (u >> LG & 31));
+        }
+    }
+    if constexpr (M::TAB_SMEM || FEW) __syncthreads();
     const uint4* in_slot = reinterpret_cast<const uint4*>(tab);            // [E/8][G] x 8
     const uint4* out_slot = reinterpret_cast<const uint4*>(tab + S);       // [E/8][G] x 8
     const uint16_t* lag_slot = tab + 2 * S;                                // [N]
-    const uint32_t* in_col = reinterpret_cast<const uint32_t*>(tab + 3 * S);   // [E/8][G]
+    const uint32_t* in_col = reinterpret_cast<const uint32_t*>(
+        tab + (FEW && M::TAB_SMEM ? 1 : 3) * S);                               // [E/8][G]
 
     // as a programmatic dependent the tables came in beside the kernel before; the row map
     // and the rows are read only after it has finished
@@ -178,7 +257,7 @@ mst_kernel(const pnce::MstLaunch p) {
     __shared__ float s_peak[16][8];                // peaks of a team's warps
 
     const int team = tid / M::TEAM, t = tid % G, sub = (tid % M::TEAM) / G;
-    float2* buf = reinterpret_cast<float2*>(mst_smem + M::TAB) + (team * M::RT + sub) * M::ROW;
+    float2* buf = reinterpret_cast<float2*>(mst_smem + (FEW ? M::TAB_FEW : M::TAB)) + (team * M::RT + sub) * M::ROW;
     const unsigned sbuf = (unsigned)__cvta_generic_to_shared(buf);
     const int teams = blockDim.x / M::TEAM;
     const long long stride = (long long)gridDim.x * teams * M::RT;
@@ -299,6 +378,23 @@ mst_kernel(const pnce::MstLaunch p) {
         }
         butterflies<E, 1, E>(v);
         team_sync<M::TEAM>(team);                  // the buffer is read: reuse it
+        if constexpr (FEW) {
+            // V_t[k] at (t + 4 k) mod G of row k: lanes of different columns, 4 or more
+            // neighbours of each, mostly meet different bank pairs
+            const unsigned rows0 = few_rows[0], rows1 = few_rows[1];
+#pragma unroll
+            for (int k = 0; k < E; ++k)
+                if ((k < 32 ? rows0 : rows1) >> (k & 31) & 1) buf[k * G + ((t + 4 * k) & (G - 1))] = v[k];
+            team_sync<M::TEAM>(team);
+            for (int c0 = 0; c0 < cols; c0 += G >> p.lg_parts) {
+                const int part = t & ((1 << p.lg_parts) - 1), c = c0 + (t >> p.lg_parts);
+                const unsigned u = few_u[c < cols ? c : 0], k = u >> LG;
+                const float2 w = column_sum<G>(buf + k * G, (int)(4 * k), u & (G - 1), part, p.lg_parts);
+                if (h && part == 0 && c < cols) h[c] = make_float2(w.x * scale, w.y * scale);
+            }
+            team_sync<M::TEAM>(team);              // the buffer takes the next row
+            continue;
+        }
 #pragma unroll
         for (int k = 0; k < E; ++k) {
             const int s = k * G + t;
@@ -340,11 +436,7 @@ mst_kernel(const pnce::MstLaunch p) {
         team_sync<M::TEAM>(team);
         if (h) {
             for (int c = t; c < cols; c += G) {
-                int lag = c;
-                if (!GRP && p.lags.mode != 0) {     // column k L + l holds lag k step + l
-                    const int k = (int)__umulhi((unsigned)c << 4, p.magic_L);
-                    lag = k * p.lags.step + (c - k * p.lags.L);
-                }
+                const int lag = GRP ? c : lag_of(p, c);
                 const float2 w = buf[lag_slot[lag]];
                 h[c] = make_float2(w.x * scale, w.y * scale);
             }
@@ -355,17 +447,26 @@ mst_kernel(const pnce::MstLaunch p) {
 
 using MstKernel = void (*)(const pnce::MstLaunch);
 
-template <int R>
-MstKernel kernel_of(bool grp, int mode) {
-    if (grp) return mode == ROUND ? mst_kernel<R, true, ROUND> : mst_kernel<R, true, PLAIN>;
-    return mode == PLAIN   ? mst_kernel<R, false, PLAIN>
-           : mode == ROUND ? mst_kernel<R, false, ROUND>
-                           : mst_kernel<R, false, CODES>;
+template <int R, bool FEW>
+MstKernel estimate_kernel(int mode) {
+    return mode == PLAIN   ? mst_kernel<R, false, PLAIN, FEW>
+           : mode == ROUND ? mst_kernel<R, false, ROUND, FEW>
+                           : mst_kernel<R, false, CODES, FEW>;
 }
 
 template <int R>
-cudaError_t launch_r(const pnce::MstTables& m, const pnce::MstLaunch& p, cudaStream_t s) {
+MstKernel kernel_of(bool grp, int mode, bool few) {
+    if (grp)
+        return mode == ROUND ? mst_kernel<R, true, ROUND, false> : mst_kernel<R, true, PLAIN, false>;
+    return few ? estimate_kernel<R, true>(mode) : estimate_kernel<R, false>(mode);
+}
+
+template <int R>
+cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t s) {
     using M = Mst<R>;
+    const bool few = p.lagvec && !p.dd && p.lags.ldH <= few_cols(R);
+    p.lg_parts = 0;                              // threads per column, 32 at most
+    while (p.lg_parts < 5 && (p.lags.ldH << (p.lg_parts + 1)) <= M::G) ++p.lg_parts;
     // rows spread over the SMs first, then over the teams of a block
     const long long teams = (p.A + M::RT - 1) / M::RT;
     const long long sms = m.num_sms;
@@ -378,14 +479,14 @@ cudaError_t launch_r(const pnce::MstTables& m, const pnce::MstLaunch& p, cudaStr
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3((unsigned)(per * M::TEAM), 1, 1);
-    cfg.dynamicSmemBytes = M::TAB + (size_t)per * M::team_bytes();
+    cfg.dynamicSmemBytes = (few ? M::TAB_FEW : M::TAB) + (size_t)per * M::team_bytes();
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = p.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel_of<R>(p.dd != nullptr, mode), p);
+    return cudaLaunchKernelEx(&cfg, kernel_of<R>(p.dd != nullptr, mode, few), p);
 }
 
 // Shared-memory limits of the kernels, and how many teams fit an SM.
@@ -398,16 +499,16 @@ cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
     if (teams > fit) teams = fit;
     const int smem = M::TAB + teams * (int)M::team_bytes();
     cudaError_t e;
-    for (const auto& km : {std::make_pair(false, (int)PLAIN), std::make_pair(false, (int)ROUND),
-                           std::make_pair(false, (int)CODES), std::make_pair(true, (int)PLAIN),
-                           std::make_pair(true, (int)ROUND)})
-        if ((e = cudaFuncSetAttribute(kernel_of<R>(km.first, km.second),
+    for (int i = 0; i < 8; ++i) {                // plain, rounding, codes, (serving: two); few
+        const int mode = i % 4 == 3 ? (i == 3 ? (int)PLAIN : (int)ROUND) : i % 4;
+        if ((e = cudaFuncSetAttribute(kernel_of<R>(i % 4 == 3, mode, i >= 4),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
             cudaSuccess)
             return e;
+    }
     m.block_teams = teams;
     int per = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of<R>(false, PLAIN),
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of<R>(false, PLAIN, false),
                                                            teams * M::TEAM, smem)) != cudaSuccess)
         return e;
     m.blocks_per_sm = per < 1 ? 1 : per;
@@ -462,12 +563,17 @@ size_t mst_table_bytes(int N) {
 }
 
 bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out) {
+    return mst_build_tables(bits_host, N, out, nullptr);
+}
+
+bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out, uint16_t* lagvec) {
     if (mst_table_bytes(N) == 0) return false;
     int r = 0;
     while ((1 << r) < N + 1) ++r;
     const int S = 1 << r, le = mst_le(r), lg = r - le, E = 1 << le, G = 1 << lg;
     std::vector<uint16_t> pos((size_t)N), lag((size_t)N);
     if (pnce_fmt_tables(bits_host, N, pos.data(), lag.data()) != PNCE_OK) return false;
+    if (lagvec) std::copy(lag.begin(), lag.end(), lagvec);
     std::vector<int> l((size_t)S), rr((size_t)S), of((size_t)S);
     std::vector<uint8_t> col;
     uint16_t* in_slot = out;
@@ -514,6 +620,7 @@ bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out) {
 cudaError_t mst_setup(MstTables& m, const uint16_t* tab_dev, int N, int num_sms,
                       int max_smem_optin) {
     m.tab = nullptr;
+    m.lagvec = nullptr;
     m.N = N;
     m.num_sms = num_sms;
     m.r = 0;
@@ -550,6 +657,7 @@ cudaError_t launch_mst(const MstTables& m, MstLaunch p, cudaStream_t s) {
                                          : 0;
     p.op_pitch = (long long)row_pitch(m.N) * elem_bytes(p.dtype);
     p.tab = m.tab;
+    p.lagvec = m.lagvec;
     p.N = m.N;
     p.invN = (float)(1.0 / (double)m.N);
     // c / L for c < 2^14 and L < 2^14 as the high word of 16 c * magic_L

@@ -25,6 +25,8 @@ struct MstLaunch {
     const void* operand = nullptr;
     const float* factors = nullptr;
     const uint16_t* tab = nullptr;
+    const uint16_t* lagvec = nullptr;
+    int lg_parts = 0;
     int N = 0;
     float invN = 0.f;
     unsigned magic_L = 0;
@@ -36,6 +38,8 @@ struct MstLaunch {
 size_t mst_table_bytes(int N);
 // Fills mst_table_bytes(N) bytes; false if the bits are no m-sequence.  May throw bad_alloc.
 bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out);
+// The same, and the vectors u_j of the lags (N entries).
+bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out, uint16_t* lagvec);
 // Describes tables that lie at tab_dev and sets the kernels' limits on the current device.
 cudaError_t mst_setup(MstTables& m, const uint16_t* tab_dev, int N, int num_sms,
                       int max_smem_optin);

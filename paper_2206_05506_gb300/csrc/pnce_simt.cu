@@ -412,7 +412,8 @@ simt_corr_warp_kernel(const uint32_t* __restrict__ bits, const float* __restrict
     }
 }
 
-// Few lags (K*L <= 32, lags contiguous): the block tile above would leave most lanes idle,
+// Few lags (K*L <= 32, lags contiguous) of a pilot that has no fast transform (no m-sequence,
+// or N below 127 or above 16383): the block tile above would leave most lanes idle,
 // and at ~2 K*L flops per 8-byte sample the work is close to the HBM roofline.  One warp
 // per received row: lane l takes the sample pairs (2p, 2p+1) for p = l, l+32, ... (four
 // pairs in flight per lane, each sample read once; one 16-byte load per pair when the
@@ -674,7 +675,7 @@ cudaError_t launch_simt_grouped(const pnce_pilot* pilot, const pnce_req_desc* dd
 cudaError_t launch_simt_bits_ex(const pnce_pilot* pilot, const float2* Y, long long y_stride,
                                 long long A, int N, const LagMap& lags, float2* H,
                                 cudaStream_t s) {
-    if (pilot->mst.tab && !(lags.mode == 0 && lags.ldH <= FEW_LAGS))
+    if (pilot->mst.tab)
         return launch_mst_rows(pilot, Y, y_stride, A, lags, PNCE_FP32_SIMT, H, s);
     if (lags.mode == 0 && lags.ldH <= FEW_LAGS)
         return launch_few_lags(pilot->ext_bits_dev, Y, y_stride, A, N, lags.ldH, lags.ldH, H, s);

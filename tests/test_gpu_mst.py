@@ -167,3 +167,59 @@ def test_traced_calls_give_the_same_bits(dtype):
     pk.trace_enable(False, dev)
     assert torch.equal(H, Ht)
     assert kinds == (["simt"] if dtype == "fp32" else ["quantize", "correlate"])
+
+
+@pytest.mark.parametrize("r, few", [(7, 8), (8, 8), (9, 8), (10, 16), (11, 32), (12, 32), (13, 32), (14, 32)])
+def test_few_lags(r, few):
+    # one lag, odd counts, the largest count of the few-lags form and the next one; rows that
+    # do not fill a team, rows with a prefix, spread shifts, rounded samples
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 2)
+    N, A, cp = bits.size, 21, 3
+    Y = _y(np.random.default_rng(r), 1, A, N + cp)
+    pilot = pk.Pilot(bits, device=dev)
+    Yd = torch.from_numpy(Y).to(dev)
+    ref = O.estimate_fft(Y[..., cp:], bits, 1, few + 1).reshape(A, -1)
+    Yc = Yd[..., cp:].contiguous()
+    for KL in (1, 2, 3, 5, few - 1, few, few + 1):
+        buf = torch.full((A * KL + 64,), complex(3.0, 3.0), dtype=torch.complex64, device=dev)
+        H = buf[32:32 + A * KL].view(1, A, 1, KL)
+        pk.estimate(Yd, pilot, 1, KL, dtype="fp32", out=H, cp_len=cp)
+        assert O.nmse(H.cpu().numpy().reshape(A, KL), ref[:, :KL]) <= TOL
+        g = torch.cat([buf[:32], buf[-32:]])
+        assert bool((g == complex(3.0, 3.0)).all()), "write outside H"
+        assert torch.equal(pk.estimate(Yc[:, 2:3].clone(), pilot, 1, KL, dtype="fp32"), H[:, 2:3])
+        for dtype in ("fp16", "e4m3"):
+            q = pk.quantize(Yc, dtype)
+            Hq = pk.correlate_quantized(q["workspace"], pilot, 1, A, 1, KL, dtype)
+            assert torch.equal(pk.estimate(Yc, pilot, 1, KL, dtype=dtype), Hq)
+            assert O.nmse(Hq.cpu().numpy(), O.estimate_quantized(Y[..., cp:], bits, 1, KL, dtype)) <= TOL
+    H = pk.estimate(Yd, pilot, 3, 2, dtype="fp32", cp_len=cp, shift_rule="spread")
+    want = O.estimate_general(Y, bits, 3, 2, cp_len=cp, shifts=np.arange(3) * (N // 3))
+    assert O.nmse(H.cpu().numpy(), want) <= TOL
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16", "e4m3", "tf32"])
+def test_rounding_at_the_edges_of_the_formats(dtype):
+    # samples half-way between two numbers of the format, down into its subnormals and below;
+    # peaks whose scale is clamped at either end, denormal rows: the quantiser's bits
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(9, 0)
+    N = bits.size
+    rng = np.random.default_rng(1)
+    x = rng.integers(1, 1 << 13, (2, N)).astype(np.float64) * 2.0 ** rng.integers(-44, 3, (2, N))
+    x *= rng.choice([-1.0, 1.0], (2, N))
+    rows = [(x[0] + 1j * x[1]) * s for s in (1.0, 2.0 ** -14, 2.0 ** -120, 2.0 ** 100, 2.0 ** 110)]
+    rows.append(_y(rng, N) * 1e-42)
+    rows.append(np.full(N, 3e38 + 1e-38j))
+    Y = torch.from_numpy(np.stack(rows).astype(np.complex64)[None]).to(dev)
+    pilot = pk.Pilot(bits, device=dev)
+    for K, L in ((3, 40), (1, 5)):
+        H = pk.estimate(Y, pilot, K, L, dtype=dtype)
+        q = pk.quantize(Y, dtype)
+        Hq = pk.correlate_quantized(q["workspace"], pilot, 1, len(rows), K, L, dtype)
+        a, b = torch.view_as_real(H), torch.view_as_real(Hq)
+        assert torch.equal(torch.isnan(a), torch.isnan(b))
+        assert torch.equal(torch.nan_to_num(a), torch.nan_to_num(b))
