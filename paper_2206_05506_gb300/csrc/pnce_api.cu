@@ -503,6 +503,23 @@ pnce_status pnce_backward(pnce_handle* h, const float* p_dev, int pilot_map, con
 
 namespace {
 
+// The address at which the GPU reads and writes `bytes` bytes of page-locked host memory at p;
+// null if they are not page-locked or not 8-byte aligned.
+void* host_mapped(const void* p, size_t bytes) {
+    cudaPointerAttributes at{}, last{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&last, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();                      // unknown pointer
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !at.devicePointer ||
+        static_cast<char*>(last.devicePointer) - static_cast<char*>(at.devicePointer) !=
+            (ptrdiff_t)bytes - 1 ||
+        ((uintptr_t)at.devicePointer & 7u))
+        return nullptr;
+    return at.devicePointer;
+}
+
 // Host pipeline layout: frames go through in chunks of fc frames, kPnceHostSlots slots of
 // (Y chunk, H chunk) so that copy-in of the next chunks and copy-out of the previous ones
 // overlap the kernels of chunk i without waiting on each other slot by slot, plus the
@@ -565,16 +582,27 @@ pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const vo
 
     // copy-out: into page-locked H_host by a kernel (it shares the host link with the
     // copy-in DMA better than a second DMA does); into pageable memory by cudaMemcpyAsync
-    unsigned char* h_mapped = nullptr;
-    {
-        cudaPointerAttributes at{};
-        if (cudaPointerGetAttributes(&at, H_host) == cudaSuccess) {
-            if (at.type == cudaMemoryTypeHost && at.devicePointer != nullptr &&
-                ((uintptr_t)at.devicePointer & 7u) == 0)
-                h_mapped = static_cast<unsigned char*>(at.devicePointer);
-        } else {
-            cudaGetLastError();                  // unknown pointer: take the copy path
-        }
+    const long long rows = (long long)F * M;
+    unsigned char* h_mapped =
+        static_cast<unsigned char*>(host_mapped(H_host, (size_t)rows * K * L * 8));
+    const char* fail_env = getenv("PNCE_TEST_HOST_FAIL_CHUNK");
+    // An m-sequence pilot and page-locked buffers: one launch that reads the rows and writes the
+    // lags over the host link itself, with no copies and no events between streams.  Few enough
+    // rows are in flight (twice the link's latency times its rate; at least one per SM) that the
+    // first results go out while the last rows come in.  The SMs read a little slower than the
+    // copy engine (196 against 207 GB/s), so large inputs with few lags keep the pipeline below.
+    // Pipeline / direct, us: 64 rows of N = 2047 with 512 lags, fp16 53 / 40, 256 rows 89 / 57,
+    // 1024 rows 148 / 118 (all rows in flight: 131), with 2047 lags 192 / 161; 4096 rows 401 /
+    // 374; 32768 rows of N = 4095, 2048 lags 5612 / 5520, 16 lags 5189 / 5473.
+    const size_t y_bytes = (size_t)rows * N * 8;
+    if (h_mapped && !fail_env && pilot->mst.tab &&
+        (dtype == PNCE_FP32_SIMT || pnce::mst_replaces_tc(pilot)) &&
+        (y_bytes <= ((size_t)128 << 20) || 4LL * K * L >= N)) {
+        if (const void* y = host_mapped(Y_host, y_bytes))
+            return from_cuda(pnce::launch_mst_rows(
+                pilot, static_cast<const float2*>(y), N, rows, pnce::lagmap_contiguous(K * L),
+                dtype, reinterpret_cast<float2*>(h_mapped), static_cast<cudaStream_t>(stream),
+                /*in_flight=*/3 << 20));
     }
 
     std::lock_guard<std::recursive_mutex> guard(h->lock);   // uses the handle's streams
@@ -589,7 +617,6 @@ pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const vo
     // Host-side fault injection for the test of the join below: PNCE_TEST_HOST_FAIL_CHUNK=i
     // makes the call give up with PNCE_ECUDA when it reaches chunk i, as a failed launch
     // or copy there would.
-    const char* fail_env = getenv("PNCE_TEST_HOST_FAIL_CHUNK");
     const long long fail_at = fail_env ? atoll(fail_env) : -1;
     auto run = [&]() -> pnce_status {
         for (cudaStream_t s : {h->s_h2d, h->s_comp, h->s_d2h})

@@ -470,11 +470,19 @@ cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t 
     // rows spread over the SMs first, then over the teams of a block
     const long long teams = (p.A + M::RT - 1) / M::RT;
     const long long sms = m.num_sms;
-    long long per = (teams + sms - 1) / sms;
+    long long most = teams;                      // teams that work at once
+    if (p.in_flight) {
+        const long long bytes = (long long)M::RT * p.N * 8;
+        most = (p.in_flight + bytes - 1) / bytes;
+        if (most < sms) most = sms;
+        if (most > teams) most = teams;
+    }
+    long long per = (most + sms - 1) / sms;
     if (per > m.block_teams) per = m.block_teams;
     long long grid = (teams + per - 1) / per;
     const long long resident = sms * (per == m.block_teams ? m.blocks_per_sm : 1);
     if (grid > resident) grid = resident;
+    if (p.in_flight && grid > (most + per - 1) / per) grid = (most + per - 1) / per;
     const int mode = p.operand ? CODES : p.dtype != PNCE_FP32_SIMT ? ROUND : PLAIN;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);

@@ -19,6 +19,7 @@ struct MstLaunch {
     const pnce_req_desc* dd = nullptr;
     const int* row_req = nullptr;
     bool pdl = false;            // a programmatic dependent of the kernel before it
+    long long in_flight = 0;     // rows in flight, in bytes, but a team per SM (0: all that fit)
     // a tensor-core dtype: the samples are rounded to it first, as the quantiser does, or,
     // with operand and factors, taken as the quantiser left them
     int dtype = PNCE_FP32_SIMT;
@@ -57,8 +58,9 @@ inline bool mst_fuses(const pnce_handle* h, const pnce_pilot* pilot) {
 // One estimate of A rows, y_stride elements apart, in one launch: FP32, or with dtype rounded.
 inline cudaError_t launch_mst_rows(const pnce_pilot* pilot, const float2* Y, long long y_stride,
                                    long long A, const LagMap& lags, int dtype, float2* H,
-                                   cudaStream_t s) {
+                                   cudaStream_t s, long long in_flight = 0) {
     MstLaunch l;
+    l.in_flight = in_flight;
     l.Y = Y;
     l.y_stride = y_stride;
     l.A = A;
