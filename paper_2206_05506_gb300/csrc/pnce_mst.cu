@@ -212,9 +212,12 @@ __device__ __forceinline__ int lag_of(const pnce::MstLaunch& p, int c) {
     return k * p.lags.step + (c - k * p.lags.L);
 }
 
-template <int R, bool GRP, int MODE, bool FEW>
-__global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
-mst_kernel(const pnce::MstLaunch p) {
+// Where the rows are: one array (ROWS), or a serving batch's requests, described by tables in
+// device memory that another kernel has checked (TABLE), or by the launch's parameters (LIST).
+enum { ROWS = 0, TABLE = 1, LIST = 2 };
+
+template <int R, int IO, int MODE, bool FEW>
+__device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::MstBatch* q) {
     using M = Mst<R>;
     constexpr int E = M::E, G = M::G, LG = M::LG, LE = M::LE, S = M::S;
     extern __shared__ __align__(16) unsigned char mst_smem[];
@@ -253,11 +256,12 @@ mst_kernel(const pnce::MstLaunch p) {
 
     // as a programmatic dependent the tables came in beside the kernel before; the row map
     // and the rows are read only after it has finished
-    if constexpr (GRP || MODE == CODES) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (IO == TABLE || MODE == CODES) asm volatile("griddepcontrol.wait;" ::: "memory");
     __shared__ float s_peak[16][8];                // peaks of a team's warps
 
     const int team = tid / M::TEAM, t = tid % G, sub = (tid % M::TEAM) / G;
-    float2* buf = reinterpret_cast<float2*>(mst_smem + (FEW ? M::TAB_FEW : M::TAB)) + (team * M::RT + sub) * M::ROW;
+    float2* buf = reinterpret_cast<float2*>(mst_smem + (FEW ? M::TAB_FEW : M::TAB)) +
+                  (team * M::RT + sub) * M::ROW;
     const unsigned sbuf = (unsigned)__cvta_generic_to_shared(buf);
     const int teams = blockDim.x / M::TEAM;
     const long long stride = (long long)gridDim.x * teams * M::RT;
@@ -269,20 +273,28 @@ mst_kernel(const pnce::MstLaunch p) {
         float2* h = nullptr;
         int cols = p.lags.ldH;
         if (row < p.A) {
-            if constexpr (GRP) {
+            if constexpr (IO == TABLE) {
                 const int b = p.row_req[row];     // a plain load: it stays behind the wait
                 if (b >= 0) {
-                    const pnce_req_desc& q = p.dd[b];
-                    cols = q.K * q.L;
-                    y = static_cast<const float2*>(q.Y) + (row - q.row_offset) * p.N;
-                    h = static_cast<float2*>(q.H) + (row - q.row_offset) * cols;
+                    const pnce_req_desc& d = p.dd[b];
+                    cols = d.K * d.L;
+                    y = static_cast<const float2*>(d.Y) + (row - d.row_offset) * p.N;
+                    h = static_cast<float2*>(d.H) + (row - d.row_offset) * cols;
                 }
+            } else if constexpr (IO == LIST) {
+                int b = 0;                         // the last request that begins at or before row
+#pragma unroll
+                for (int d = pnce::kMstBatchMax / 2; d; d >>= 1)
+                    if (b + d < q->n && q->row0[b + d] <= row) b += d;
+                cols = q->cols[b];
+                y = q->Y[b] + (row - q->row0[b]) * p.N;
+                h = q->H[b] + (row - q->row0[b]) * cols;
             } else {
                 y = p.Y + row * p.y_stride;
                 h = p.H + row * p.lags.ldH;
             }
         }
-        if constexpr (GRP) {                       // a team without a row has nothing to do
+        if constexpr (IO == TABLE) {               // a team without a row has nothing to do
             if (M::RT == 1 ? y == nullptr : __all_sync(0xffffffffu, y == nullptr)) continue;
         }
         if constexpr (MODE == CODES) {
@@ -323,7 +335,7 @@ mst_kernel(const pnce::MstLaunch p) {
             }
         }
         if constexpr (MODE != CODES) asm volatile("cp.async.wait_all;\n" ::: "memory");
-        if constexpr (!GRP && MODE != CODES) {
+        if constexpr (IO == ROWS && MODE != CODES) {
             if (t == 0 && row + stride < p.A) prefetch_l2(y + stride * p.y_stride, p.N);
         }
         team_sync<M::TEAM>(team);
@@ -384,7 +396,8 @@ mst_kernel(const pnce::MstLaunch p) {
             const unsigned rows0 = few_rows[0], rows1 = few_rows[1];
 #pragma unroll
             for (int k = 0; k < E; ++k)
-                if ((k < 32 ? rows0 : rows1) >> (k & 31) & 1) buf[k * G + ((t + 4 * k) & (G - 1))] = v[k];
+                if ((k < 32 ? rows0 : rows1) >> (k & 31) & 1)
+                    buf[k * G + ((t + 4 * k) & (G - 1))] = v[k];
             team_sync<M::TEAM>(team);
             for (int c0 = 0; c0 < cols; c0 += G >> p.lg_parts) {
                 const int part = t & ((1 << p.lg_parts) - 1), c = c0 + (t >> p.lg_parts);
@@ -392,79 +405,98 @@ mst_kernel(const pnce::MstLaunch p) {
                 const float2 w = column_sum<G>(buf + k * G, (int)(4 * k), u & (G - 1), part, p.lg_parts);
                 if (h && part == 0 && c < cols) h[c] = make_float2(w.x * scale, w.y * scale);
             }
-            team_sync<M::TEAM>(team);              // the buffer takes the next row
-            continue;
-        }
+        } else {
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int s = k * G + t;
-            buf[s + (s >> M::L2)] = v[k];
-        }
-        team_sync<M::TEAM>(team);
-        // second pass: the low L2 levels in registers, the X above them by lane shuffles
+            for (int k = 0; k < E; ++k) {
+                const int s = k * G + t;
+                buf[s + (s >> M::L2)] = v[k];
+            }
+            team_sync<M::TEAM>(team);
+            // second pass: the low L2 levels in registers, the X above them by lane shuffles
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int s = pass2_entry(LE, LG, t, k);
-            v[k] = buf[s + (s >> M::L2)];
-        }
-        butterflies<E, 1, (1 << M::L2)>(v);
-        if constexpr (M::X > 0) {
+            for (int k = 0; k < E; ++k) {
+                const int s = pass2_entry(LE, LG, t, k);
+                v[k] = buf[s + (s >> M::L2)];
+            }
+            butterflies<E, 1, (1 << M::L2)>(v);
+            if constexpr (M::X > 0) {
 #pragma unroll
-            for (int d = 1; d < (1 << M::X); d <<= 1) {
-                const float sg = (t & d) ? -1.f : 1.f;
+                for (int d = 1; d < (1 << M::X); d <<= 1) {
+                    const float sg = (t & d) ? -1.f : 1.f;
 #pragma unroll
-                for (int k = 0; k < E; ++k) {
-                    const float px = __shfl_xor_sync(0xffffffffu, v[k].x, d);
-                    const float py = __shfl_xor_sync(0xffffffffu, v[k].y, d);
-                    v[k] = make_float2(fmaf(sg, v[k].x, px), fmaf(sg, v[k].y, py));
+                    for (int k = 0; k < E; ++k) {
+                        const float px = __shfl_xor_sync(0xffffffffu, v[k].x, d);
+                        const float py = __shfl_xor_sync(0xffffffffu, v[k].y, d);
+                        v[k] = make_float2(fmaf(sg, v[k].x, px), fmaf(sg, v[k].y, py));
+                    }
                 }
             }
-        }
-        team_sync<M::TEAM>(team);
-        // out: only the lines of lags that are wanted (contiguous lags), all of them otherwise
-        const unsigned lim = p.lags.mode == 0 ? (unsigned)((cols + 15) & ~15) : (unsigned)S;
+            team_sync<M::TEAM>(team);
+            // out: only the lines of lags that are wanted (contiguous lags), all of them otherwise
+            const unsigned lim = p.lags.mode == 0 ? (unsigned)((cols + 15) & ~15) : (unsigned)S;
 #pragma unroll
-        for (int k8 = 0; k8 < E / 8; ++k8) {
-            const uint4 q = out_slot[k8 * G + t];
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+            for (int k8 = 0; k8 < E / 8; ++k8) {
+                const uint4 q = out_slot[k8 * G + t];
+                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const unsigned slot = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu;
-                if (slot < lim) buf[slot] = v[8 * k8 + e];
+                for (int e = 0; e < 8; ++e) {
+                    const unsigned slot = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu;
+                    if (slot < lim) buf[slot] = v[8 * k8 + e];
+                }
             }
-        }
-        team_sync<M::TEAM>(team);
-        if (h) {
-            for (int c = t; c < cols; c += G) {
-                const int lag = GRP ? c : lag_of(p, c);
-                const float2 w = buf[lag_slot[lag]];
-                h[c] = make_float2(w.x * scale, w.y * scale);
+            team_sync<M::TEAM>(team);
+            if (h) {
+                for (int c = t; c < cols; c += G) {
+                    const int lag = IO != ROWS ? c : lag_of(p, c);
+                    const float2 w = buf[lag_slot[lag]];
+                    h[c] = make_float2(w.x * scale, w.y * scale);
+                }
             }
         }
         team_sync<M::TEAM>(team);                  // the buffer takes the next row
     }
 }
 
+template <int R, int IO, int MODE, bool FEW>
+__global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
+mst_kernel(const __grid_constant__ pnce::MstLaunch p) {
+    mst_rows<R, IO, MODE, FEW>(p, nullptr);
+}
+
+template <int R, int MODE>
+__global__ void __launch_bounds__(Mst<R>::MAXT, Mst<R>::MINB)
+mst_batch_kernel(const __grid_constant__ pnce::MstLaunch p,
+                 const __grid_constant__ pnce::MstBatch q) {
+    mst_rows<R, LIST, MODE, false>(p, &q);
+}
+
 using MstKernel = void (*)(const pnce::MstLaunch);
+using MstBatchKernel = void (*)(const pnce::MstLaunch, const pnce::MstBatch);
 
 template <int R, bool FEW>
 MstKernel estimate_kernel(int mode) {
-    return mode == PLAIN   ? mst_kernel<R, false, PLAIN, FEW>
-           : mode == ROUND ? mst_kernel<R, false, ROUND, FEW>
-                           : mst_kernel<R, false, CODES, FEW>;
+    return mode == PLAIN   ? mst_kernel<R, ROWS, PLAIN, FEW>
+           : mode == ROUND ? mst_kernel<R, ROWS, ROUND, FEW>
+                           : mst_kernel<R, ROWS, CODES, FEW>;
 }
 
 template <int R>
-MstKernel kernel_of(bool grp, int mode, bool few) {
-    if (grp)
-        return mode == ROUND ? mst_kernel<R, true, ROUND, false> : mst_kernel<R, true, PLAIN, false>;
+MstKernel kernel_of(bool table, int mode, bool few) {
+    if (table)
+        return mode == ROUND ? mst_kernel<R, TABLE, ROUND, false>
+                             : mst_kernel<R, TABLE, PLAIN, false>;
     return few ? estimate_kernel<R, true>(mode) : estimate_kernel<R, false>(mode);
+}
+
+template <int R>
+MstBatchKernel batch_kernel_of(int mode) {
+    return mode == ROUND ? mst_batch_kernel<R, ROUND> : mst_batch_kernel<R, PLAIN>;
 }
 
 template <int R>
 cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t s) {
     using M = Mst<R>;
-    const bool few = p.lagvec && !p.dd && p.lags.ldH <= few_cols(R);
+    const bool few = p.lagvec && !p.dd && !p.batch && p.lags.ldH <= few_cols(R);
     p.lg_parts = 0;                              // threads per column, 32 at most
     while (p.lg_parts < 5 && (p.lags.ldH << (p.lg_parts + 1)) <= M::G) ++p.lg_parts;
     // rows spread over the SMs first, then over the teams of a block
@@ -494,6 +526,7 @@ cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = p.pdl ? 1 : 0;
+    if (p.batch) return cudaLaunchKernelEx(&cfg, batch_kernel_of<R>(mode), p, *p.batch);
     return cudaLaunchKernelEx(&cfg, kernel_of<R>(p.dd != nullptr, mode, few), p);
 }
 
@@ -514,6 +547,11 @@ cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
             cudaSuccess)
             return e;
     }
+    for (int mode : {(int)PLAIN, (int)ROUND})
+        if ((e = cudaFuncSetAttribute(batch_kernel_of<R>(mode),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
+            cudaSuccess)
+            return e;
     m.block_teams = teams;
     int per = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of<R>(false, PLAIN, false),

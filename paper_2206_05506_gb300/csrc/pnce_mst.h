@@ -7,6 +7,17 @@ namespace pnce {
 
 constexpr int kMstMinR = 7, kMstMaxR = 14;
 
+// A serving batch of up to kMstBatchMax requests, passed with the launch: request i has the
+// rows row0[i] .. row0[i + 1) of the batch (row0[0] = 0, ascending; the last up to the launch's
+// A), N samples each from Y[i] on, and cols[i] = K*L lags per row from H[i] on.
+constexpr int kMstBatchMax = 64;                 // a power of two
+struct MstBatch {
+    int n;
+    int row0[kMstBatchMax], cols[kMstBatchMax];
+    const float2* Y[kMstBatchMax];
+    float2* H[kMstBatchMax];
+};
+
 // One launch: rows of y_stride elements at Y (p.lags says which lags go where in H), or,
 // with dd, the rows of a serving batch, read from and written to the requests' buffers
 // (contiguous lags, K*L of each request).  What follows `factors` is filled in.
@@ -18,6 +29,7 @@ struct MstLaunch {
     float2* H = nullptr;
     const pnce_req_desc* dd = nullptr;
     const int* row_req = nullptr;
+    const MstBatch* batch = nullptr;   // in host memory; in the place of Y, H, dd and row_req
     bool pdl = false;            // a programmatic dependent of the kernel before it
     long long in_flight = 0;     // rows in flight, in bytes, but a team per SM (0: all that fit)
     // a tensor-core dtype: the samples are rounded to it first, as the quantiser does, or,

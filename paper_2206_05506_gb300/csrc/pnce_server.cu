@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "pnce_internal.h"
+#include "pnce_mst.h"
 
 namespace {
 
@@ -414,8 +415,51 @@ struct CudaExec {
         const double pitch = (double)((r.N + 63) / 64 * 64);
         return (double)r.M * (8.0 * r.N + 2.0 * elt * pitch + 8.0 * kl_class(r.K * r.L, r.N));
     }
+    // A batch whose pilot has a fast transform: one launch with the requests in its parameters,
+    // without the graph, the descriptor table and the kernel that checks it (the requests are
+    // checked here).  False: not such a batch.  48 requests, 5792 rows, 64 MB over the link:
+    // the loop 468 -> 439 us on FP32, 457 -> 435 on fp16 (four slots).
+    bool launch_listed(int slot, int N, int klc, const std::vector<const pnce_serve_req*>& rs,
+                       long long rows, cudaError_t* err) {
+        const auto it = sv->pilots.find(N);
+        const int dtype = pnce::resolve_dtype(sv->dtype, klc);
+        if (it == sv->pilots.end() || rs.size() > (size_t)pnce::kMstBatchMax ||
+            rows > 0x7fffffffLL || !it->second->mst.tab ||
+            !(dtype == PNCE_FP32_SIMT || pnce::mst_replaces_tc(it->second)))
+            return false;
+        pnce::MstBatch b;
+        b.n = (int)rs.size();
+        int off = 0;
+        for (int k = 0; k < b.n; ++k) {
+            const pnce_serve_req& r = *rs[(size_t)k];
+            if ((uintptr_t)r.Y & 7u || (uintptr_t)r.H & 7u) return false;
+            b.row0[k] = off;
+            b.cols[k] = r.K * r.L;
+            b.Y[k] = static_cast<const float2*>(r.Y);
+            b.H[k] = static_cast<float2*>(r.H);
+            off += r.M;
+        }
+        pnce::MstLaunch l;
+        l.A = rows;
+        l.lags = pnce::lagmap_contiguous(klc);
+        l.batch = &b;
+        l.dtype = dtype;
+        *err = pnce::launch_mst(it->second->mst, l, sv->streams[(size_t)slot]);
+        return true;
+    }
     bool launch(int slot, int N, int klc, const std::vector<const pnce_serve_req*>& rs,
                 long long rows, int* status) {
+        cudaError_t e = cudaSuccess;
+        if (launch_listed(slot, N, klc, rs, rows, &e)) {
+            if (e != cudaSuccess ||
+                cudaEventRecord(sv->events[(size_t)slot], sv->streams[(size_t)slot]) !=
+                    cudaSuccess) {
+                cudaGetLastError();
+                *status = PNCE_ECUDA;
+                return false;
+            }
+            return true;
+        }
         ServeShape* sh = nullptr;
         const pnce_status st = get_shape(sv, slot, N, klc, capacity_for(rows), &sh);
         if (st != PNCE_OK) {

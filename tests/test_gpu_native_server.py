@@ -179,3 +179,35 @@ def test_native_online_session(setup):
         assert O.nmse(_result(out, r)[None], ref) <= TOL["fp16"]
     nat.start()                                       # a new session once all are reported
     assert nat.open_requests() == 0
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "fp32"])
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 130])
+def test_many_requests_in_one_batch(setup, dtype, n):
+    # batches of uneven small requests, at and above the 64 that go with the launch: the
+    # single estimates' bits, nothing written between the results
+    import paper_2206_05506_gb300 as pk
+    serve, _, _ = setup
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator().manual_seed(n)
+    for N in (127, 511):
+        shapes = [(1 + i % 3, 1 + i % 2, 1 + 7 * (i % 5)) for i in range(n)]
+        ys = [torch.randn(M, N, dtype=torch.complex64, generator=gen).pin_memory() for M, _, _ in shapes]
+        out = torch.full((sum(M * K * L + 1 for M, K, L in shapes),), complex(3.0, 3.0),
+                         dtype=torch.complex64).pin_memory()
+        nat = serve.NativeServer(S.pilot_bits, device=dev, dtype=dtype, slots=2, max_batch_rows=256)
+        reqs, off = [], 0
+        for i, ((M, K, L), y) in enumerate(zip(shapes, ys)):
+            reqs.append(serve.Request(i, 0.0, M, N, K, L, y.data_ptr(), out.data_ptr() + 8 * off))
+            off += M * K * L + 1
+        st = nat.run(reqs)
+        assert st["failed"] == 0 and st["batches"] <= 2
+        pilot, off = nat.pilot(N), 0
+        for (M, K, L), y in zip(shapes, ys):
+            H = pk.estimate(y.to(dev)[None], pilot, K, L, dtype=dtype).cpu()
+            got = out[off:off + M * K * L].view(1, M, K, L)
+            # (up to 8 lags a single estimate sums in another order)
+            assert torch.equal(got, H) if K * L > 8 else O.nmse(got.numpy(), H.numpy()) <= 1e-11
+            off += M * K * L
+            assert out[off] == complex(3.0, 3.0)
+            off += 1
