@@ -17,7 +17,9 @@ dtype: "fp32" (exact FP32 on the CUDA cores), or "tf32" / "fp16" / "bf16" / "e4m
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import threading
+from operator import index
 
 import numpy as np
 import torch
@@ -46,7 +48,19 @@ def _dt(dtype) -> int:
 
 
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    # the handle itself; a torch.cuda.Stream object around it costs over a microsecond
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
+def _call(what: str, device, fn, *args) -> None:
+    """fn(*args) with `device` current; a status other than PNCE_OK raises PnceError."""
+    if torch._C._cuda_getDevice() == device.index:
+        st = fn(*args)
+    else:
+        with torch.cuda.device(device):
+            st = fn(*args)
+    if st:
+        check(st, what)
 
 
 def _ptr(t) -> int | None:
@@ -87,6 +101,10 @@ _contexts: dict[int, Context] = {}
 
 
 def context(device=None) -> Context:
+    if isinstance(device, torch.device) and device.type == "cuda":
+        ctx = _contexts.get(device.index)
+        if ctx is not None:
+            return ctx
     dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
     idx = dev.index if dev.index is not None else torch.cuda.current_device()
     with _ctx_lock:
@@ -203,14 +221,18 @@ def estimate_fmt(Y: torch.Tensor, fmt: "FmtPilot", K: int, L: int, out=None) -> 
         raise ValueError("Y's N differs from the transform's")
     dev = Y.device
     H = _out_or_new(out, (F, M, K, L), dev)
-    with torch.cuda.device(dev):
-        check(lib().pnce_estimate_fmt(fmt.ctx.handle, fmt.handle, Y.data_ptr(), F, M, N, K, L,
-                                      H.data_ptr(), _stream(dev)), "pnce_estimate_fmt")
+    _call("pnce_estimate_fmt", dev, lib().pnce_estimate_fmt, fmt.ctx.handle, fmt.handle,
+          Y.data_ptr(), F, M, N, K, L, H.data_ptr(), _stream(dev))
     return H
 
 
 def workspace_size(F, M, N, K, L, dtype) -> int:
-    return int(lib().pnce_workspace_size(F, M, N, K, L, _dt(dtype)))
+    return _workspace_size(*map(index, (F, M, N, K, L)), _dt(dtype))
+
+
+@functools.lru_cache(maxsize=1024)
+def _workspace_size(F, M, N, K, L, dt) -> int:
+    return int(lib().pnce_workspace_size(F, M, N, K, L, dt))
 
 
 def grouped_workspace_size(rows, N, kl_max, dtype) -> int:
@@ -233,11 +255,21 @@ def estimate_grouped(pilot: "Pilot", descs_ptr: int, nreq: int, rows: int, kl_ma
 
 
 def backward_workspace_size(F, M, N, K, L) -> int:
+    return _backward_workspace_size(*map(index, (F, M, N, K, L)))
+
+
+@functools.lru_cache(maxsize=1024)
+def _backward_workspace_size(F, M, N, K, L) -> int:
     return int(lib().pnce_backward_workspace_size(F, M, N, K, L))
 
 
 def host_workspace_size(F, M, N, K, L, dtype) -> int:
-    return int(lib().pnce_host_workspace_size(F, M, N, K, L, _dt(dtype)))
+    return _host_workspace_size(*map(index, (F, M, N, K, L)), _dt(dtype))
+
+
+@functools.lru_cache(maxsize=1024)
+def _host_workspace_size(F, M, N, K, L, dt) -> int:
+    return int(lib().pnce_host_workspace_size(F, M, N, K, L, dt))
 
 
 _ws_cache: dict[tuple, torch.Tensor] = {}
@@ -329,16 +361,14 @@ def estimate(Y: torch.Tensor, pilot: Pilot, K: int, L: int, dtype="fp32", out=No
     ws = _check_workspace(workspace, dev, need) if workspace is not None \
         else _workspace(dev, need)
     nbytes = 0 if ws is None else ws.numel() * ws.element_size()
-    with torch.cuda.device(dev):
-        if cp_len == 0 and shift_rule == "kl":
-            check(lib().pnce_estimate(pilot.ctx.handle, pilot.handle, Y.data_ptr(), F, M, N, K,
-                                      L, dt, _ptr(ws), nbytes, H.data_ptr(), _stream(dev)),
-                  "pnce_estimate")
-        else:
-            opts = _lib.FrameOpts(cp_len, SHIFT_RULES[shift_rule])
-            check(lib().pnce_estimate_ex(pilot.ctx.handle, pilot.handle, Y.data_ptr(), F, M, N,
-                                         K, L, dt, C.byref(opts), _ptr(ws), nbytes, H.data_ptr(),
-                                         _stream(dev)), "pnce_estimate_ex")
+    if cp_len == 0 and shift_rule == "kl":
+        _call("pnce_estimate", dev, lib().pnce_estimate, pilot.ctx.handle, pilot.handle,
+              Y.data_ptr(), F, M, N, K, L, dt, _ptr(ws), nbytes, H.data_ptr(), _stream(dev))
+    else:
+        opts = _lib.FrameOpts(cp_len, SHIFT_RULES[shift_rule])
+        _call("pnce_estimate_ex", dev, lib().pnce_estimate_ex, pilot.ctx.handle, pilot.handle,
+              Y.data_ptr(), F, M, N, K, L, dt, C.byref(opts), _ptr(ws), nbytes, H.data_ptr(),
+              _stream(dev))
     return H
 
 
@@ -415,11 +445,9 @@ def estimate_real_pilot(Y: torch.Tensor, p: torch.Tensor, K: int, L: int, out=No
         raise ValueError("p must be a contiguous float32 tensor [N] on Y's device")
     dev = Y.device
     H = _out_or_new(out, (F, M, K, L), dev)
-    with torch.cuda.device(dev):
-        check(lib().pnce_estimate_real_pilot(context(dev).handle, p.data_ptr(),
-                                             PILOT_MAPS[pilot_map], Y.data_ptr(), F, M, N, K, L,
-                                             H.data_ptr(), _stream(dev)),
-              "pnce_estimate_real_pilot")
+    _call("pnce_estimate_real_pilot", dev, lib().pnce_estimate_real_pilot, context(dev).handle,
+          p.data_ptr(), PILOT_MAPS[pilot_map], Y.data_ptr(), F, M, N, K, L, H.data_ptr(),
+          _stream(dev))
     return H
 
 
@@ -437,12 +465,9 @@ def backward(p: torch.Tensor, Y: torch.Tensor, G: torch.Tensor, K: int, L: int,
     dp = torch.empty(N, dtype=torch.float32, device=dev) if need_dp else None
     need = backward_workspace_size(F, M, N, K, L) if need_dp else 0
     ws = _workspace(dev, need, key="bwd")
-    with torch.cuda.device(dev):
-        check(lib().pnce_backward(context(dev).handle, p.data_ptr(), PILOT_MAPS[pilot_map],
-                                  Y.data_ptr(), G.data_ptr(), F, M, N, K, L, _ptr(dY), _ptr(dp),
-                                  _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
-                                  _stream(dev)),
-              "pnce_backward")
+    _call("pnce_backward", dev, lib().pnce_backward, context(dev).handle, p.data_ptr(),
+          PILOT_MAPS[pilot_map], Y.data_ptr(), G.data_ptr(), F, M, N, K, L, _ptr(dY), _ptr(dp),
+          _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(), _stream(dev))
     return dY, dp
 
 
@@ -465,11 +490,8 @@ def estimate_host(Y_host: torch.Tensor, pilot: Pilot, K: int, L: int, dtype="fp3
     need = host_workspace_size(F, M, N, K, L, dt)
     ws = _check_workspace(workspace, dev, need) if workspace is not None \
         else _workspace(dev, need, key="host")
-    with torch.cuda.device(dev):
-        s = _stream(dev)
-        check(lib().pnce_estimate_host(pilot.ctx.handle, pilot.handle, Y_host.data_ptr(), F, M,
-                                       N, K, L, dt, _ptr(ws),
-                                       0 if ws is None else ws.numel() * ws.element_size(),
-                                       H.data_ptr(), s), "pnce_estimate_host")
-        torch.cuda.current_stream(dev).synchronize()
+    _call("pnce_estimate_host", dev, lib().pnce_estimate_host, pilot.ctx.handle, pilot.handle,
+          Y_host.data_ptr(), F, M, N, K, L, dt, _ptr(ws),
+          0 if ws is None else ws.numel() * ws.element_size(), H.data_ptr(), _stream(dev))
+    torch.cuda.current_stream(dev).synchronize()
     return H

@@ -367,10 +367,12 @@ def _native_stats(requests: list, out: np.ndarray, batches: int) -> dict:
     """Write the run's times into the Request objects and summarise them as Server.stats
     does."""
     ok = out["status"] == 0
-    for r, o in zip(requests, out):
-        r.t_admit, r.t_launch, r.t_done = float(o["t_admit"]), float(o["t_launch"]), float(o["t_done"])
-        r.batch = int(o["batch"])
-        r.error = "" if o["status"] == 0 else f"status {int(o['status'])}"
+    # lists first: a field of one record read through NumPy costs as much as ten of a list
+    for r, ta, tl, td, b, st in zip(requests, out["t_admit"].tolist(), out["t_launch"].tolist(),
+                                    out["t_done"].tolist(), out["batch"].tolist(),
+                                    out["status"].tolist()):
+        r.t_admit, r.t_launch, r.t_done, r.batch = ta, tl, td, b
+        r.error = "" if st == 0 else f"status {st}"
     if not ok.any():
         return {"requests": 0, "failed": int((~ok).sum())}
     t_arr = np.array([r.t_arrival for r in requests])
@@ -379,11 +381,12 @@ def _native_stats(requests: list, out: np.ndarray, batches: int) -> dict:
     lat = (out["t_done"] - t_arr)[ok]
     span = max(float(out["t_done"][ok].max() - t_arr[ok].min()), 1e-9)
     launched = out["batch"] >= 0
+    p50, p99 = np.percentile(lat, (50, 99))
     rows = np.bincount(out["batch"][launched], weights=M[launched], minlength=batches)[:batches]
     return {"requests": int(lat.size), "batches": int(batches),
             "mean_batch_rows": float(rows.mean()) if batches else 0.0,
-            "p50_ms": float(np.percentile(lat, 50) * 1e3),
-            "p99_ms": float(np.percentile(lat, 99) * 1e3),
+            "p50_ms": float(p50 * 1e3),
+            "p99_ms": float(p99 * 1e3),
             "max_ms": float(lat.max() * 1e3),
             "frames_per_s": lat.size / span, "taps_per_s": float((M * KL)[ok].sum()) / span,
             "failed": int((~ok).sum())}
