@@ -60,11 +60,12 @@ struct Mst {
     static constexpr int ROW = S + (S >> L2);            // entries of a row's buffer, padded
     // tables in shared memory; for r >= 13 they are read from global memory
     static constexpr bool TAB_SMEM = R <= 12;
-    static constexpr int TAB = TAB_SMEM ? S * 6 + S / 2 : 0;
-    static constexpr int TAB_FEW = TAB_SMEM ? S * 2 + S / 2 : 0;     // the few-lags kernel's
+    static constexpr int TAB = TAB_SMEM ? (S * 6 + S / 2 + 127) / 128 * 128 : 0;
+    static constexpr int TAB_FEW = TAB_SMEM ? (S * 2 + S / 2 + 127) / 128 * 128 : 0;   // of FEW
     // most threads per block and most blocks per SM (registers: 2 E + about 40 each)
     static constexpr int MAXT = R >= 14 ? 256 : R >= 11 ? 384 : R >= 9 ? 640 : 512;
     static constexpr int MINB = R >= 9 ? 1 : 2;
+    static_assert(ROW * sizeof(float2) % 128 == 0, "row buffers are 128-byte aligned");
     static constexpr size_t team_bytes() { return (size_t)RT * ROW * sizeof(float2); }
 };
 
@@ -93,6 +94,13 @@ __device__ __forceinline__ void prefetch_l2(const float2* row, int n) {
     const uintptr_t a = ((uintptr_t)row + 15) & ~(uintptr_t)15;
     const unsigned bytes = (unsigned)((uintptr_t)(row + n) - a) & ~15u;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
+}
+
+// the largest magnitude; a NaN is left out
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
 // butterfly levels on register distances FIRST, 2 FIRST, .. < LAST
@@ -124,7 +132,9 @@ __device__ __forceinline__ void round_entries(float2 (&v)[E], float sc) {
 // than the format's smallest, leaves v 2^s rounded to even at the format's last place (a NaN
 // stays one).  Conversions to and from the formats seem to issue at 16 a clock per SM and held
 // the kernel up: 65536 rows of N = 4095, 2048 lags, fp16 0.78 -> 0.65 ms; e4m3, 32768 rows, 0.347
-// -> 0.337 ms.  (bf16 and tf32 need one and two conversions per sample: 0.33 ms both.)
+// -> 0.337 ms.  (bf16 and tf32 need one and two conversions per sample.)  Adding and clamping
+// the exponent in one instruction, the peak by three-way maxima and the colour or-ed into the
+// address of the first pass's reads: 0.643 -> 0.615 ms and 0.336 -> 0.323 ms.
 template <int DT, int E>
 __device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
     constexpr int D = DT == PNCE_FP16 ? 13 : 20, EMIN = DT == PNCE_FP16 ? -14 : -6;
@@ -133,8 +143,8 @@ __device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
 #pragma unroll
     for (int k = 0; k < E; ++k) {
         const float2 big = make_float2(
-            __int_as_float(max((__float_as_int(v[k].x) & 0x7f800000) + add, least)),
-            __int_as_float(max((__float_as_int(v[k].y) & 0x7f800000) + add, least)));
+            __int_as_float(__viaddmax_s32(__float_as_int(v[k].x) & 0x7f800000, add, least)),
+            __int_as_float(__viaddmax_s32(__float_as_int(v[k].y) & 0x7f800000, add, least)));
         v[k] = __ffma2_rn(big, m1, __ffma2_rn(v[k], sc2, big));
     }
 }
@@ -143,7 +153,7 @@ __device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
 // registers to what the quantiser would store (each value is exact in FP32), so the step is
 // one pass over Y with no operand in memory, and the sums keep all FP32 bits that the tensor
 // cores truncate.  One pass against quantise + tensor-core correlation: 65536 rows of
-// N = 4095, 2048 lags, fp16 1.43 -> 0.65 ms, e4m3 (32768 rows) 0.485 -> 0.337 ms; 8192 rows of
+// N = 4095, 2048 lags, fp16 1.43 -> 0.615 ms, e4m3 (32768 rows) 0.485 -> 0.32 ms; 8192 rows of
 // N = 1023, 512 lags, tf32 60 -> 27 us; relative error of the sums at N = 4095, fp16,
 // 1.4e-6 -> 1e-7.  CODES reads an operand that the quantiser has stored (traced calls, the
 // separate correlation step): the same bits.
@@ -220,17 +230,17 @@ template <int R, int IO, int MODE, bool FEW>
 __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::MstBatch* q) {
     using M = Mst<R>;
     constexpr int E = M::E, G = M::G, LG = M::LG, LE = M::LE, S = M::S;
-    extern __shared__ __align__(16) unsigned char mst_smem[];
+    extern __shared__ __align__(128) unsigned char mst_smem[];
     const int tid = threadIdx.x;
     const uint16_t* tab;
     if constexpr (M::TAB_SMEM) {
         const uint4* src = reinterpret_cast<const uint4*>(p.tab);
         uint4* dst = reinterpret_cast<uint4*>(mst_smem);
         if constexpr (FEW) {
-            for (int i = tid; i < M::TAB_FEW / 16; i += blockDim.x)
+            for (int i = tid; i < (S * 2 + S / 2) / 16; i += blockDim.x)
                 dst[i] = __ldg(src + (i < S / 8 ? i : i + S / 4));
         } else {
-            for (int i = tid; i < M::TAB / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+            for (int i = tid; i < (S * 6 + S / 2) / 16; i += blockDim.x) dst[i] = __ldg(src + i);
         }
         tab = reinterpret_cast<const uint16_t*>(mst_smem);
     } else {
@@ -348,7 +358,12 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int k = 8 * k8 + e;
-                v[k] = buf[k * G + (t & ~15) + ((c >> (4 * e)) & 15u)];
+                // 8 x the colour, or-ed into the address of the line: rows are 128-byte aligned
+                const uint32_t off = (e == 0 ? c << 3 : c >> (4 * e - 3)) & 0x78u;
+                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];"
+                             : "=f"(v[k].x), "=f"(v[k].y)
+                             : "r"(((sbuf + 8 * (t & ~15)) | off) + 8 * G * k)
+                             : "memory");
             }
         }
         float scale = p.invN;
@@ -360,7 +375,7 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
             float m = 0.f;
             if (p.target != 0) {                   // NaN parts are left out, as fmaxf does
 #pragma unroll
-                for (int k = 0; k < E; ++k) m = fmaxf(m, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
+                for (int k = 0; k < E; ++k) m = max3_abs(m, v[k].x, v[k].y);
 #pragma unroll
                 for (int o = (G < 32 ? G : 32) / 2; o; o >>= 1)
                     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
