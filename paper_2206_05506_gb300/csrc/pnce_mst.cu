@@ -264,9 +264,13 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
     const uint32_t* in_col = reinterpret_cast<const uint32_t*>(
         tab + (FEW && M::TAB_SMEM ? 1 : 3) * S);                               // [E/8][G]
 
-    // as a programmatic dependent the tables came in beside the kernel before; the row map
-    // and the rows are read only after it has finished
-    if constexpr (IO == TABLE || MODE == CODES) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // as a programmatic dependent the tables came in beside the kernel before; everything else
+    // is read and written only after it has finished.  Estimates that follow each other in a
+    // stream overlap their launches and their last rows this way: 4736 rows of N = 2047, 512 lags
+    // 26.8 -> 25.1 us; 8192 rows of N = 1023 22.5 -> 21.9.  (No block of the next grid can keep
+    // one of this grid waiting: the grids are no larger than what is resident.)
+    if constexpr (IO == ROWS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (IO != LIST) asm volatile("griddepcontrol.wait;" ::: "memory");
     __shared__ float s_peak[16][8];                // peaks of a team's warps
 
     const int team = tid / M::TEAM, t = tid % G, sub = (tid % M::TEAM) / G;
@@ -540,7 +544,7 @@ cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t 
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = p.pdl ? 1 : 0;
+    cfg.numAttrs = p.pdl || !(p.dd || p.batch) ? 1 : 0;
     if (p.batch) return cudaLaunchKernelEx(&cfg, batch_kernel_of<R>(mode), p, *p.batch);
     return cudaLaunchKernelEx(&cfg, kernel_of<R>(p.dd != nullptr, mode, few), p);
 }
