@@ -182,7 +182,10 @@ pnce_status pnce_quantize(pnce_handle* h, const void* Y_dev, int F, int M, int N
 
 /*
  * Correlation of an operand already quantised into workspace_dev by pnce_quantize (same F,
- * M, N, dtype): the second step of pnce_estimate alone, with the same bits.  Lets callers time or overlap the quantisation separately.
+ * M, N, dtype): the second step of pnce_estimate alone, with the same bits, except that
+ * operands of more than 2^22 samples with few lags (K*L times the bytes of a code at most 1024) go
+ * to the tensor cores, whose accumulation rounds differently.  Lets callers time or overlap the
+ * quantisation separately.
  */
 pnce_status pnce_correlate_quantized(pnce_handle* h, const pnce_pilot* pilot,
                                      int F, int M, int N, int K, int L, int dtype,

@@ -350,10 +350,17 @@ pnce_status pnce_correlate_quantized(pnce_handle* h, const pnce_pilot* pilot, in
     if (pilot->device != h->device || pilot->N != N) return PNCE_ESTATE;
     const pnce::QuantLayout lay = pnce::quant_layout(A, N, dtype);
     void* ws = const_cast<void*>(workspace_dev);
+    // Large operands with few lags go to the tensor cores, which read the operand at the memory's
+    // rate there; the transform spends its time on all 2^r entries whatever K*L.  Tensor cores /
+    // transform, us, 65536 rows of N = 4095: 16 lags fp16 163 / 340, e4m3 88 / 334, tf32 331 /
+    // 433; 2048 lags 952 / 551, 532 / 539, 1983 / 683; 8192 rows of N = 1023, 512 lags 19.6 /
+    // 20.1, 16.9 / 20.3, 31 / 24; 64 rows of N = 2047, 512 lags, fp16 16.3 / 10.2.
+    const bool tensor_cores = (long long)K * L * pnce::elem_bytes(dtype) <= 1024 &&
+                              A * N > (1LL << 22);
     pnce::TraceScope tr(h, static_cast<cudaStream_t>(stream), pnce::TRACE_CORRELATE);
     return pnce::launch_tc(h, pilot, A, N, K * L, dtype, pnce::ws_operand(ws, lay),
                            pnce::ws_factors(ws, lay), static_cast<float2*>(H_dev),
-                           static_cast<cudaStream_t>(stream));
+                           static_cast<cudaStream_t>(stream), /*pdl=*/false, tensor_cores);
 }
 
 pnce_status pnce_estimate(pnce_handle* h, const pnce_pilot* pilot, const void* Y_dev, int F,

@@ -196,13 +196,15 @@ cudaError_t launch_quantize_grouped(const pnce_req_desc* dd, const int* row_req,
 // status: PNCE_OK, or PNCE_ECUDA / PNCE_EUNSUPPORTED.  pdl: launch as a programmatic
 // dependent of the kernel before it on the stream (the kernel's set-up -- barriers, TMEM,
 // the resident pilot operand -- then overlaps that kernel's tail; it waits for it before
-// touching the operand).
+// touching the operand).  An m-sequence pilot's operand goes to the fast transform instead
+// (pnce_mst.cu), unless tensor_cores is set.
 pnce_status launch_tc(const pnce_handle* h, const pnce_pilot* pilot, long long A, int N,
                       int KL, int dtype, const void* operand, const float* factors, float2* H,
-                      cudaStream_t s, bool pdl = false);
+                      cudaStream_t s, bool pdl = false, bool tensor_cores = false);
 pnce_status launch_tc_ex(const pnce_handle* h, const pnce_pilot* pilot, long long A, int N,
                          const LagMap& lags, int dtype, const void* operand,
-                         const float* factors, float2* H, cudaStream_t s, bool pdl = false);
+                         const float* factors, float2* H, cudaStream_t s, bool pdl = false,
+                         bool tensor_cores = false);
 // the two pointers of a workspace laid out by quant_layout
 inline void* ws_operand(void* ws, const QuantLayout& l) {
     return static_cast<unsigned char*>(ws) + l.a_offset;

@@ -162,6 +162,49 @@ __device__ __forceinline__ void round_small(float2 (&v)[E], float sc, int se) {
 // (ROUND), or codes that the quantiser has stored (CODES).
 enum { PLAIN = 0, ROUND = 1, CODES = 2 };
 
+// A row of stored codes into its buffer: the loads of up to 32 samples first (the registers are
+// free at this point), then their conversions; the team's next row is asked of L2.  With the
+// format looked up per sample, and so one sample's loads at a time, 65536 rows of N = 4095 with
+// 2048 lags took 4.9 ms in fp16; now 0.55
+// (e4m3 0.54, bf16 0.55, tf32 0.68).
+template <int R, int DT>
+__device__ __forceinline__ void load_codes(const pnce::MstLaunch& p, long long row,
+                                           long long stride, const uint4* in_slot, float2* buf,
+                                           int t) {
+    using M = Mst<R>;
+    using T = typename pnce::Fmt<DT>::T;
+    constexpr int E = M::E, G = M::G, B = E < 32 ? E : 32;
+    const char* op = static_cast<const char*>(p.operand);
+    const T* re = reinterpret_cast<const T*>(op + pnce::operand_row(row, 0) * p.op_pitch);
+    const T* im = reinterpret_cast<const T*>(op + pnce::operand_row(row, 1) * p.op_pitch);
+    if (t < 2 && row + stride < p.A) {
+        const void* next = op + pnce::operand_row(row + stride, t) * p.op_pitch;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(next),
+                     "r"((unsigned)p.op_pitch) : "memory");
+    }
+#pragma unroll
+    for (int b = 0; b < E; b += B) {
+        T cr[B], ci[B];
+#pragma unroll
+        for (int e = 0; e < B; ++e) {              // (rows are padded: sample N can be read)
+            cr[e] = __ldg(re + t + G * (b + e));
+            ci[e] = __ldg(im + t + G * (b + e));
+        }
+#pragma unroll
+        for (int e8 = 0; e8 < B; e8 += 8) {
+            const uint4 q = in_slot[(b + e8) / 8 * G + t];
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float2 x = pnce::decode<DT>(cr[e8 + e], ci[e8 + e]);
+                if (b + e8 + e == E - 1 && t + G * (E - 1) >= p.N)
+                    x = make_float2(0.f, 0.f);     // entry 0 of X is zero
+                buf[(e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu] = x;
+            }
+        }
+    }
+}
+
 // Few lags (FEW): the second pass and the exchange before it would form all 2^r sums for a
 // handful.  Instead the registers' sums V_t[k] of the wanted rows k (the upper bits of the
 // columns' vectors u_j: at most one row per column) are left in the buffer, and P threads per
@@ -313,25 +356,11 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
         }
         if constexpr (MODE == CODES) {
             if (row < p.A) {
-                const unsigned char* op = static_cast<const unsigned char*>(p.operand);
-                const unsigned char* re = op + pnce::operand_row(row, 0) * p.op_pitch;
-                const unsigned char* im = op + pnce::operand_row(row, 1) * p.op_pitch;
-#pragma unroll
-                for (int i8 = 0; i8 < E / 8; ++i8) {
-                    const uint4 q = in_slot[i8 * G + t];
-                    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-                    float2 x[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int n = t + G * (8 * i8 + e);
-                        x[e] = make_float2(0.f, 0.f);           // entry 0 of X is zero
-                        if (n < p.N)
-                            x[e] = make_float2(pnce::decode(p.dtype, re, n),
-                                               pnce::decode(p.dtype, im, n));
-                    }
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        buf[(e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xffffu] = x[e];
+                switch (p.dtype) {
+                    case PNCE_FP16: load_codes<R, PNCE_FP16>(p, row, stride, in_slot, buf, t); break;
+                    case PNCE_BF16: load_codes<R, PNCE_BF16>(p, row, stride, in_slot, buf, t); break;
+                    case PNCE_TF32: load_codes<R, PNCE_TF32>(p, row, stride, in_slot, buf, t); break;
+                    default: load_codes<R, PNCE_FP8E4M3>(p, row, stride, in_slot, buf, t); break;
                 }
             }
         } else if (y) {

@@ -59,19 +59,18 @@ __device__ __forceinline__ float2 round_through(float2 v) {
             __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)to_e4m3x2(v.x, v.y), __NV_E4M3)));
 }
 
-// one stored code as a number
-__device__ __forceinline__ float decode(int dtype, const void* row, int n) {
-    switch (dtype) {
-        case PNCE_FP16:
-            return __half2float(__ushort_as_half(__ldg(static_cast<const uint16_t*>(row) + n)));
-        case PNCE_BF16:
-            return __bfloat162float(
-                __ushort_as_bfloat16(__ldg(static_cast<const uint16_t*>(row) + n)));
-        case PNCE_TF32: return __ldg(static_cast<const float*>(row) + n);
-        default:
-            return __half2float(__half(__nv_cvt_fp8_to_halfraw(
-                (__nv_fp8_storage_t)__ldg(static_cast<const uint8_t*>(row) + n), __NV_E4M3)));
-    }
+// one complex sample from its stored codes
+template <int DT>
+__device__ __forceinline__ float2 decode(typename Fmt<DT>::T re, typename Fmt<DT>::T im) {
+    if constexpr (DT == PNCE_FP16)
+        return make_float2(__half2float(__ushort_as_half(re)), __half2float(__ushort_as_half(im)));
+    else if constexpr (DT == PNCE_BF16)
+        return make_float2(__uint_as_float((uint32_t)re << 16), __uint_as_float((uint32_t)im << 16));
+    else if constexpr (DT == PNCE_TF32)
+        return make_float2(__uint_as_float(re), __uint_as_float(im));
+    else
+        return __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(
+            (__nv_fp8x2_storage_t)(re | (uint16_t)im << 8), __NV_E4M3)));
 }
 
 }  // namespace pnce

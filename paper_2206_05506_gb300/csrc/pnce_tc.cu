@@ -1813,9 +1813,9 @@ namespace pnce {
 
 pnce_status launch_tc_ex(const pnce_handle* h, const pnce_pilot* pilot, long long A, int N,
                          const LagMap& lm, int dtype, const void* operand, const float* factors,
-                         float2* H, cudaStream_t s, bool pdl) {
+                         float2* H, cudaStream_t s, bool pdl, bool tensor_cores) {
     if (!(h->cc_major == 10 && h->cc_minor == 3)) return PNCE_EUNSUPPORTED;
-    if (mst_replaces_tc(pilot)) {
+    if (!tensor_cores && mst_replaces_tc(pilot)) {
         MstLaunch l;
         l.A = A;
         l.lags = lm;
@@ -1841,9 +1841,9 @@ pnce_status launch_tc_ex(const pnce_handle* h, const pnce_pilot* pilot, long lon
 
 pnce_status launch_tc(const pnce_handle* h, const pnce_pilot* pilot, long long A, int N, int KL,
                       int dtype, const void* operand, const float* factors, float2* H,
-                      cudaStream_t s, bool pdl) {
+                      cudaStream_t s, bool pdl, bool tensor_cores) {
     return launch_tc_ex(h, pilot, A, N, lagmap_contiguous(KL), dtype, operand, factors, H, s,
-                        pdl);
+                        pdl, tensor_cores);
 }
 
 }  // namespace pnce

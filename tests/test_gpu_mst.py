@@ -223,3 +223,20 @@ def test_rounding_at_the_edges_of_the_formats(dtype):
         a, b = torch.view_as_real(H), torch.view_as_real(Hq)
         assert torch.equal(torch.isnan(a), torch.isnan(b))
         assert torch.equal(torch.nan_to_num(a), torch.nan_to_num(b))
+
+
+@pytest.mark.parametrize("dtype, KL", [("fp16", 500), ("bf16", 30), ("e4m3", 500), ("tf32", 250)])
+def test_large_operands_with_few_lags(dtype, KL):
+    # the correlation step alone, on either side of 2^22 samples: the transform's bits below, the
+    # tensor cores above (their truncated accumulation: relative error 1e-5, NMSE 1e-10)
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(9, 0)
+    N, pilot = bits.size, pk.Pilot(bits, device=dev)
+    for A in (8207, 8209):                       # 8208 x 511 > 2^22 > 8207 x 511
+        Y = torch.randn(1, A, N, dtype=torch.complex64, device=dev, generator=torch.Generator(dev).manual_seed(A))
+        H = pk.estimate(Y, pilot, 1, KL, dtype=dtype)
+        q = pk.quantize(Y, dtype)
+        Hq = pk.correlate_quantized(q["workspace"], pilot, 1, A, 1, KL, dtype)
+        assert torch.equal(H, Hq) if A * N < 1 << 22 else O.nmse(Hq.cpu().numpy(), H.cpu().numpy()) <= 1e-10
+    assert pk.get_status(dev) == 0
