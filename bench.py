@@ -1,16 +1,15 @@
 """Benchmark: PN-correlation channel estimation throughput on GB300.
 
-One step = one pnce_estimate call over one batch: per-antenna quantisation of the
-received blocks, then the tensor-core correlation with its epilogue, on synthetic
-received blocks shaped like the precision workload (M=128 antennas, N=4095 m-sequence,
-K=16 transmitters x L=128 taps, 512 frames, SNR 0/10/20/30 dB), inputs resident in
-HBM.  The library's tracing records CUDA events around each kernel it
-launches, on the stream the kernel runs on; the correlation kernels' durations give the
-roofline figure.
+One step = one pnce_estimate call over one batch, on synthetic received blocks shaped like
+the precision workload (M=128 antennas, N=4095 m-sequence, K=16 transmitters x L=128 taps,
+512 frames, SNR 0/10/20/30 dB), inputs resident in HBM: one launch, which rounds each
+antenna's samples to the scaled format and correlates them by the fast m-sequence transform.
 
 value      CIR taps estimated per second (one tap = one complex H entry), all ranks
 e2e        the same metric through pnce_estimate_host: host (pinned) Y in, host H out
-roofline   the correlation kernel against the measured dense tensor peak for its dtype
+roofline   that launch against the measured copy bandwidth; with it, the tensor-core
+           correlation (the path of other pilots) against the measured dense peak of its
+           dtype, timed by the library's tracing (CUDA events around each kernel)
 cpu_baseline  the FP64 oracle (Toeplitz product through numpy's BLAS) on a frame sample
 
 Multi-GPU: frames are independent, so every rank estimates its own batch with no
@@ -395,46 +394,27 @@ def run_serving_batch(dev, replays: int):
                 e1.synchronize()
                 if i >= 20:
                     ts.append(e0.elapsed_time(e1) * 1e3)
-            # the correlation kernel's own time: eager runs of the same batch with the
-            # library's tracing on (no dependent-launch overlap, so the kernel is alone)
-            graph, shape.graph = shape.graph, None
-            pk.trace_enable(True, dev)
-            pk.trace_read(dev)
-            for i in range(20):
-                shape.run(eng, 0, [serve.Request(0, 0.0, M, N, K, L,
-                                                 pool[i % blocks].data_ptr(), H.data_ptr())])
-            torch.cuda.synchronize()
-            kind = "correlate" if dtype != "fp32" else "simt"
-            kt = [t for k, t in pk.trace_read(dev) if k == kind]
-            pk.trace_enable(False, dev)
-            shape.graph = graph
-            kern_us = float(np.median(kt)) * 1e3 if kt else None
-            flops = 4.0 * N * M * K * L                          # the request's own taps
-            peaks, _ = load_peaks()
             row = {"gpu_us_median": float(np.median(ts)),
                    "gpu_us_p90": float(np.percentile(ts, 90)), "replays": replays,
-                   "bytes_in": M * N * 8, "bytes_out": M * K * L * 8,
-                   "correlation_kernel_us": kern_us}
-            if kern_us:
-                achieved = flops / (kern_us * 1e-6) / 1e12
-                sms = torch.cuda.get_device_properties(dev).multi_processor_count
-                peak = (peaks["bf16_tflops"] * DTYPE_RATIO[dtype] if dtype != "fp32"
-                        else sms * 128 * 2 * 2070e6 / 1e12)
-                row["correlation_roofline"] = {
-                    "bound": "tensor" if dtype != "fp32" else "alu", "achieved": achieved,
-                    "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "note": "a lone request: a few CTAs, bound by set-up and drain latency"}
+                   "bytes_in": M * N * 8, "bytes_out": M * K * L * 8}
             out[f"{dtype}_m{M}_n{N}_kl{K * L}"] = row
             del eng
         del pool
     return out
 
 
+def transform_roofline(w, ms, peaks, peak_src):
+    """The fast m-sequence transform against the memory: every sample read once, every lag
+    written once, in ms per launch."""
+    gbs = 8.0 * w.F * w.M * (w.N + w.K * w.L) / (ms / 1e3) / 1e9
+    return {"bound": "hbm", "kernel": "mst_kernel", "achieved": gbs, "peak": peaks["hbm_gbs"],
+            "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"], "peak_source": f"{peak_src} copy"}
+
+
 def run_paper_scale(dev, ref=None, reps: int = 50):
     """The paper-scale workload (M = 64, N = 1023, K = 8, L = 64, 128 frames, SNR 0/10/20
-    dB): the plain FP32 SIMT path against the TF32 tensor-core path (and fp16), each with
-    its step time, throughput, the roofline fraction of its correlation kernel and, given
-    the oracle's estimate `ref`, its NMSE overall and per SNR."""
+    dB) in FP32, TF32 and fp16, each with its step time, throughput, the roofline fraction
+    of its one kernel and, given the oracle's estimate `ref`, its NMSE overall and per SNR."""
     import torch
 
     import paper_2206_05506_gb300 as pk
@@ -446,8 +426,6 @@ def run_paper_scale(dev, ref=None, reps: int = 50):
     H = torch.empty((w.F, w.M, w.K, w.L), dtype=torch.complex64, device=dev)
     peaks, peak_src = load_peaks()
     taps = w.F * w.M * w.K * w.L
-    flops = 4.0 * w.F * w.M * w.N * w.K * w.L
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
     stream = torch.cuda.current_stream(dev)
     out = {"workload": w.name}
     for dt in ("fp32", "tf32", "fp16"):
@@ -456,8 +434,6 @@ def run_paper_scale(dev, ref=None, reps: int = 50):
         for _ in range(5):
             pk.estimate(Yd, pilot, w.K, w.L, dtype=dt, out=H, workspace=ws)
         torch.cuda.synchronize()
-        pk.trace_enable(True, dev)
-        pk.trace_read(dev)
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record(stream)
@@ -465,26 +441,9 @@ def run_paper_scale(dev, ref=None, reps: int = 50):
             pk.estimate(Yd, pilot, w.K, w.L, dtype=dt, out=H, workspace=ws)
         e1.record(stream)
         torch.cuda.synchronize()
-        tr = pk.trace_read(dev)
-        pk.trace_enable(False, dev)
         ms = e0.elapsed_time(e1) / reps
-        kind = "simt" if dt == "fp32" else "correlate"
-        kern_ms = float(np.median([t for k, t in tr if k == kind]))
-        q_ms = [t for k, t in tr if k == "quantize"]
-        achieved = flops / (kern_ms / 1e3) / 1e12
-        if dt == "fp32":
-            peak = sms * 128 * 2 * 2070.0 * 1e6 / 1e12
-            roof = {"bound": "alu", "kernel": "simt_corr_kernel", "achieved": achieved,
-                    "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flop x 2070 MHz"}
-        else:
-            peak = peaks["bf16_tflops"] * DTYPE_RATIO[dt]
-            roof = {"bound": "tensor", "kernel": "tc_corr_kernel", "achieved": achieved,
-                    "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "peak_source": f"{peak_src} burst bf16 x {DTYPE_RATIO[dt]}"}
         row = {"ms_per_step": ms, "value": taps / (ms / 1e3), "unit": "taps/s",
-               "kernel_ms": kern_ms,
-               "quantize_ms": float(np.median(q_ms)) if q_ms else 0.0, "roofline": roof}
+               "roofline": transform_roofline(w, ms, peaks, peak_src)}
         if ref is not None:
             row.update(nmse_stats(H.cpu().numpy(), ref, w.frame_snr()))
         out[dt] = row
@@ -609,7 +568,7 @@ def run_layouts(dev, pilot, Y, K, L, taps_per_step, reps: int = 30):
 
 def run_small_case(dev, ref=None, calls: int = 200):
     """Launch-latency case: one frame of 8 antennas, N = 127, K = 2, L = 16 (8 KB in, 2 KB
-    out), FP32 (the transform's few-lags form).  Per call: the kernel's device time (the
+    out), FP32 (the transform kernel).  Per call: the kernel's device time (the
     library's trace events around the launch), the host wall time of the call and its
     synchronisation, and end to end from page-locked host memory (pnce_estimate_host: copy
     in, estimate, copy out).  ref: the oracle's result (from oracle_references) or None."""
@@ -816,15 +775,13 @@ def main():
     stream = torch.cuda.current_stream(dev)
 
     def step():
-        # the product call (quantise, then correlate; PNCE_OVERLAP_CHUNKS would overlap them)
+        # the product call: one launch of the transform kernel per step
         pk.estimate(Y, pilot, K, L, dtype=dt, out=H, workspace=ws)
 
-    pk.trace_enable(True, dev)
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
     assert pk.get_status(dev) == 0
-    pk.trace_read(dev)
 
     e_start = torch.cuda.Event(enable_timing=True)
     e_end = torch.cuda.Event(enable_timing=True)
@@ -841,33 +798,31 @@ def main():
     clocks.mark_end()
     barrier()
     clk = clocks.stop()
-    trace = pk.trace_read(dev)       # (kind, ms) of every kernel launched in the timed region
-    pk.trace_enable(False, dev)
     total_ms = max_over_ranks(e_start.elapsed_time(e_end), world, dev)
     assert pk.get_status(dev) == 0
-    main_kind = "simt" if dt == "fp32" else "correlate"
-    corr_ms = [ms for kind, ms in trace if kind == main_kind]
-    quant_ms = [ms for kind, ms in trace if kind == "quantize"]
-    launches = len(trace)
-    nch = max(1, len(corr_ms) // args.steps)
+    launches = args.steps            # one per estimate (m-sequence pilot, no switch set)
 
     taps_per_step = F * M * K * L
     value = taps_per_step * args.steps * world / (total_ms / 1e3)
 
-    # the correlation kernel alone (operand quantised once, nothing running beside it), for
-    # comparison with its in-step duration above
-    alone_ms = None
+    # the paper's method on the same batch: quantiser and tensor-core correlation, one by one
+    tc_ms = {}
     if dt != "fp32":
-        q = pk.quantize(Y, dt, workspace=ws)
+        os.environ["PNCE_TC_FORCE"] = "1"
         for _ in range(3):
+            pk.quantize(Y, dt, workspace=ws)
             pk.correlate_quantized(ws, pilot, F, M, K, L, dt, out=H)
         pk.trace_enable(True, dev)
         pk.trace_read(dev)
         for _ in range(20):
+            pk.quantize(Y, dt, workspace=ws)
             pk.correlate_quantized(ws, pilot, F, M, K, L, dt, out=H)
-        alone_ms = float(np.mean([ms for _, ms in pk.trace_read(dev)]))
+        for kind, ms in pk.trace_read(dev):
+            tc_ms.setdefault(kind, []).append(ms)
         pk.trace_enable(False, dev)
-        del q
+        del os.environ["PNCE_TC_FORCE"]
+        tc_ms = {kind: float(np.mean(v)) for kind, v in tc_ms.items()}
+        step()                       # H: the product call's result again
 
     # ---- end to end through the host-buffer entry point
     H_pin = torch.empty((F, M, K, L), dtype=torch.complex64, pin_memory=True)
@@ -902,34 +857,17 @@ def main():
             dist.destroy_process_group()
         return
 
-    # ---- roofline of the correlation kernel
+    # ---- roofline of the step's kernel (the step is that one launch)
     peaks, peak_src = load_peaks()
-    # per correlation launch (one frame chunk): real GEMM of 2 Fc M rows x N x KL, 2 flop
-    # per MAC (the SIMT path does the same 2 FMA per complex sample and lag)
-    flops = 4.0 * (F / nch) * M * N * K * L
-    kern_ms = float(np.mean(corr_ms))
-    if dt == "fp32":
-        # FP32 CUDA-core peak: 152 SMs x 128 FMA lanes x 2 flop x SM clock (2070 MHz max)
-        sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        mhz = (clk or {}).get("sm_mhz") or 2070.0
-        peak = sms * 128 * 2 * mhz * 1e6 / 1e12
-        achieved = flops / (kern_ms / 1e3) / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "simt_corr_kernel",
-                "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flop x {mhz:.0f} MHz"}
-    else:
-        long_region = total_ms > 1000.0
-        base = peaks["bf16_tflops_sustained" if long_region else "bf16_tflops"]
-        peak = base * DTYPE_RATIO[dt]
-        achieved = flops / (kern_ms / 1e3) / 1e12
-        alone = 4.0 * F * M * N * K * L / (alone_ms / 1e3) / 1e12
-        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak,
-                "kernel_alone": {"ms_per_launch": alone_ms, "frames_per_launch": F,
-                                 "achieved": alone, "frac": alone / peak},
-                "traffic": traffic_from_profile(w.name, dt, F / nch),
-                "kernel": "tc_corr_kernel", "peak_source":
-                f"{peak_src} {'sustained' if long_region else 'burst'} bf16 x {DTYPE_RATIO[dt]}"}
+    kern_ms = total_ms / args.steps
+    roof = transform_roofline(w, kern_ms, peaks, peak_src)
+    if tc_ms:
+        tflops = 4.0 * F * M * N * K * L / (tc_ms["correlate"] / 1e3) / 1e12
+        peak = peaks["bf16_tflops"] * DTYPE_RATIO[dt]
+        roof["tensor_cores"] = {"kernel": "tc_corr_kernel", "ms_per_launch": tc_ms["correlate"],
+                                "quantize_ms": tc_ms["quantize"], "achieved": tflops,
+                                "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
+                                "traffic": traffic_from_profile(w.name, dt, F)}
 
     # ---- CPU baseline (FP64 oracle) on a frame sample, plus accuracy of those frames.  It
     # and the legs below describe the single-GPU configuration: they run at N = 1 only
@@ -1003,10 +941,7 @@ def main():
         "config": {"workload": w.name, "frames": F, "M": M, "N": N, "K": K, "L": L,
                    "snr_db": list(w.snr_db), "parallelism": f"frames x{world}",
                    "l2": f"inputs larger than L2 ({Y.numel() * 8 / 1e9:.2f} GB Y per step)"},
-        "breakdown_ms": {"correlate_per_launch": kern_ms,
-                         "correlate_launches_per_step": nch,
-                         "quantize_per_launch": float(np.mean(quant_ms)) if quant_ms else 0.0,
-                         "traced_kernels": launches},
+        "breakdown_ms": {"estimate_per_launch": kern_ms, "launches_per_step": 1},
         "roofline": roof,
         "e2e": {"value": e2e_value, "unit": "taps/s",
                 "h2d_bytes_per_step": int(Y_pin.numel() * 8),
