@@ -110,23 +110,23 @@ pnce_status pnce_fmt_tables(const uint32_t* bits_host, int N, uint16_t* pos, uin
     if ((1LL << r) != (long long)N + 1 || r < 2 || r > MAX_R) return PNCE_EINVAL;
     std::vector<uint8_t> b((size_t)N);
     for (int n = 0; n < N; ++n) b[(size_t)n] = (uint8_t)((bits_host[n >> 5] >> (n & 31)) & 1u);
-    // windows: distinct and nonzero
+    // windows: distinct and nonzero; each is the one before shifted by a bit
     std::vector<int> inv((size_t)1 << r, -1);
-    for (int n = 0; n < N; ++n) {
-        uint32_t s = 0;
-        for (int i = 0; i < r; ++i) s |= (uint32_t)b[(size_t)((n + i) % N)] << i;
+    uint32_t s = 0;
+    for (int i = 0; i < r; ++i) s |= (uint32_t)b[(size_t)i] << i;
+    for (int n = 0, next = r; n < N; ++n) {
         if (s == 0 || inv[s] >= 0) return PNCE_EINVAL;
         inv[s] = n;
         pos[n] = (uint16_t)s;
+        s = (s >> 1) | (uint32_t)b[(size_t)next] << (r - 1);
+        if (++next == N) next = 0;
     }
-    // u_j from the unit windows
-    for (int j = 0; j < N; ++j) {
-        uint32_t u = 0;
-        for (int i = 0; i < r; ++i) {
-            const long long ni = inv[(size_t)1 << i];
-            u |= (uint32_t)b[(size_t)(((ni - j) % N + N) % N)] << i;
-        }
-        lagvec[j] = (uint16_t)u;
+    // u_j from the unit windows: bit i of u_j is bit n_i - j (mod N) of the pilot
+    for (int j = 0; j < N; ++j) lagvec[j] = 0;
+    for (int i = 0; i < r; ++i) {
+        const int ni = inv[(size_t)1 << i];
+        for (int j = 0; j <= ni; ++j) lagvec[j] |= (uint16_t)(b[(size_t)(ni - j)] << i);
+        for (int j = ni + 1; j < N; ++j) lagvec[j] |= (uint16_t)(b[(size_t)(ni - j + N)] << i);
     }
     // the recurrence the windows imply must hold over the whole period: with j = N - r,
     // b[n + r] = <u_j, s_n> for every n (then every u_j is right, by linearity)

@@ -616,22 +616,19 @@ cudaError_t setup_r(pnce::MstTables& m, int max_smem_optin) {
 void colour16(const std::vector<int>& l, const std::vector<int>& r, std::vector<uint8_t>& col) {
     const int S = (int)l.size(), V = S / 16;
     col.assign((size_t)S, 0);
-    std::vector<int> pl((size_t)S), pr((size_t)S), open((size_t)V * 16);
+    std::vector<int> pl((size_t)S + 1), pr((size_t)S + 1), open((size_t)V * 16);
     std::vector<int8_t> half((size_t)S);
     for (int level = 0; level < 4; ++level) {
         for (int side = 0; side < 2; ++side) {
             const std::vector<int>& v = side ? r : l;
             std::vector<int>& p = side ? pr : pl;
             std::fill(open.begin(), open.end(), -1);
-            for (int e = 0; e < S; ++e) {
+            for (int e = 0; e < S; ++e) {          // (no branch: it would be a coin toss)
                 int& o = open[(size_t)v[(size_t)e] * 16 + col[(size_t)e]];
-                if (o < 0) {
-                    o = e;
-                } else {
-                    p[(size_t)e] = o;
-                    p[(size_t)o] = e;
-                    o = -1;
-                }
+                const int first = o;
+                p[(size_t)e] = first;              // the first of a pair: set by the second
+                p[(size_t)(first < 0 ? S : first)] = e;
+                o = first < 0 ? e : -1;
             }
         }
         std::fill(half.begin(), half.end(), (int8_t)-1);
@@ -683,7 +680,7 @@ bool mst_build_tables(const uint32_t* bits_host, int N, uint16_t* out, uint16_t*
     colour16(l, rr, col);
     for (int n = 0; n < S; ++n) {
         const int s = n < N ? pos[(size_t)n] : 0;
-        const int i = n / G, t = n % G;
+        const int i = n >> lg, t = n & (G - 1);
         in_slot[((i / 8) * G + t) * 8 + i % 8] = (uint16_t)((s & ~15) | col[(size_t)n]);
         of[(size_t)s] = col[(size_t)n];
     }

@@ -240,3 +240,26 @@ def test_large_operands_with_few_lags(dtype, KL):
         Hq = pk.correlate_quantized(q["workspace"], pilot, 1, A, 1, KL, dtype)
         assert torch.equal(H, Hq) if A * N < 1 << 22 else O.nmse(Hq.cpu().numpy(), H.cpu().numpy()) <= 1e-10
     assert pk.get_status(dev) == 0
+
+
+@pytest.mark.parametrize("r, KL", [(7, 8), (10, 3), (12, 32)])
+def test_few_lags_of_samples_that_are_not_numbers(r, KL):
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    bits = mseq.mseq_bits(r, 0)
+    N = bits.size
+    Y = _y(np.random.default_rng(r), 1, 5, N)
+    Y[0, 0, 3] = complex(np.nan, 1.0)
+    Y[0, 1, 4] = complex(2.0, np.inf)
+    Y[0, 2, N - 1] = complex(-np.inf, 0.5)
+    Y[0, 3, [5, 9]] = complex(np.inf, 1.0)
+    H = pk.estimate(torch.from_numpy(Y).to(dev), pk.Pilot(bits, device=dev), 1, KL,
+                    dtype="fp32").cpu().numpy()[0, :, 0]
+    P = np.stack([np.roll(1.0 - 2.0 * bits, j) for j in range(KL)], axis=1)
+    with np.errstate(invalid="ignore"):
+        want = np.stack([(Y[0].real[:, :, None] * P).sum(1), (Y[0].imag[:, :, None] * P).sum(1)])
+    for got, w in ((H.real, want[0]), (H.imag, want[1])):
+        assert np.array_equal(np.isnan(got), np.isnan(w))
+        inf, fine = np.isinf(w), np.isfinite(w)
+        assert np.array_equal(np.isinf(got), inf) and np.array_equal(np.sign(got[inf]), np.sign(w[inf]))
+        assert np.allclose(got[fine], w[fine] / N, rtol=0, atol=1e-5)
