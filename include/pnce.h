@@ -237,8 +237,10 @@ pnce_status pnce_backward(pnce_handle* h, const float* pilot_dev, int pilot_map,
  * buffers should be page-locked for the copies to be asynchronous.  Y comes in by
  * cudaMemcpyAsync; H goes out by a copy kernel storing into H_host when H_host is
  * page-locked memory known to CUDA (it shares the host link with the inbound copy better
- * than a second DMA does), by cudaMemcpyAsync otherwise.  Calls on the same handle are
- * serialised on the handle's pipeline streams.
+ * than a second DMA does), by cudaMemcpyAsync otherwise.  With an m-sequence pilot and both
+ * buffers page-locked, inputs of up to 128 MB (of any size if K*L >= N / 4) take one launch on
+ * the caller's stream that reads and writes them over the link; the workspace is not used.
+ * Pipelined calls on the same handle are serialised on the handle's streams.
  */
 size_t pnce_host_workspace_size(int F, int M, int N, int K, int L, int dtype);
 pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const void* Y_host,

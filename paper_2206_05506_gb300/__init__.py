@@ -12,7 +12,9 @@ cyclic shifts k*L of one m-sequence, Sec. II-B).
     H = estimate(Y, pilot, K, L, dtype="fp16")  # Y: complex64 CUDA tensor [F, M, N]
 
 dtype: "fp32" (exact FP32 on the CUDA cores), or "tf32" / "fp16" / "bf16" / "e4m3"
-(per-antenna power-of-two scaled operand, tensor cores, FP32 accumulation).
+(per-antenna power-of-two scaled operand, FP32 accumulation).  m-sequence pilots of 127 to
+16383 samples take the fast m-sequence transform in every dtype, one launch; other pilots the
+dense FP32 kernels or the tensor cores.
 """
 from __future__ import annotations
 
@@ -416,7 +418,9 @@ def quantize(Y: torch.Tensor, dtype, workspace=None, want_power=False):
 
 
 def correlate_quantized(workspace: torch.Tensor, pilot: Pilot, F, M, K, L, dtype, out=None):
-    """Tensor-core correlation of an operand already produced by quantize()."""
+    """Correlation of an operand already produced by quantize(): estimate()'s bits for
+    m-sequence pilots that take the transform, but for large operands with few lags, which
+    the tensor cores correlate (pnce_correlate_quantized)."""
     dt = _dt(dtype)
     dev = pilot.device
     N = pilot.N
