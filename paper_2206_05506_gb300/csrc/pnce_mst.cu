@@ -322,6 +322,16 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
     const unsigned sbuf = (unsigned)__cvta_generic_to_shared(buf);
     const int teams = blockDim.x / M::TEAM;
     const long long stride = (long long)gridDim.x * teams * M::RT;
+    // Teams that start together load together and then add together.  Where a row is several
+    // microseconds of work (r >= 11) and each team has two or more, half of the teams start 2 us
+    // later: the other half's first rows still keep the memory busy, and from then on one half
+    // loads while the other adds.  us without / with: N = 2047, 4736 rows of 4 x 128 spread lags
+    // 31.7 / 29.8, 5473 rows of 1024 lags 32.0 / 29.6; N = 4095, 65536 rows of 2048 lags 552 /
+    // 545, fp16 615 / 606, 2737 rows 34.8 / 32.1, 32768 rows of 16 lags 177.5 / 174.2 (1.5 to 5 us
+    // are alike).  Shorter rows lose: N = 1023 fp16 1 %, N = 127 with 5 lags 5-13 %.
+    if constexpr (R >= 11 && IO == ROWS && MODE != CODES) {
+        if (team >= teams / 2 && 2 * stride <= p.A) __nanosleep(2200);
+    }
 
     for (long long row0 = ((long long)blockIdx.x * teams + team) * M::RT; row0 < p.A;
          row0 += stride) {
