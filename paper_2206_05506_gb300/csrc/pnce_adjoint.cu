@@ -233,7 +233,7 @@ cudaError_t launch_dp(const DpGrid& g, const float2* G, const float2* Y, long lo
 namespace pnce {
 
 size_t backward_workspace(long long A, int N, int KL) {
-    if (fft_adjoint_applies(N, KL)) return fft_adjoint_workspace(A, N, KL);
+    if (fft_dp_applies(N, KL)) return fft_adjoint_workspace(A, N, KL);
     const DpGrid g = dp_grid(A, N);
     return round_up((size_t)(g.P * g.Q) * (size_t)g.QT * sizeof(float), 256);
 }
@@ -242,11 +242,14 @@ cudaError_t launch_backward(const float* p, bool tanh_map, const float2* Y, cons
                             long long A, int N, int KL, float2* dY, float* dp, void* ws,
                             size_t ws_bytes, cudaStream_t s) {
     if (dp && ws_bytes < backward_workspace(A, N, KL)) return cudaErrorInvalidValue;
-    if (fft_adjoint_applies(N, KL)) return launch_fft_adjoint(p, tanh_map, G, Y, A, N, KL, dY, dp, ws, s);
+    if (fft_adjoint_applies(N, KL))
+        return launch_fft_adjoint(p, tanh_map, G, Y, A, N, KL, dY, dp, ws, s);
     if (dY) {
         cudaError_t e = launch_adjoint_dy(p, tanh_map, G, A, N, KL, dY, s);
         if (e != cudaSuccess) return e;
     }
+    if (dp && fft_dp_applies(N, KL))
+        return launch_fft_adjoint(p, tanh_map, G, Y, A, N, KL, nullptr, dp, ws, s);
     if (dp) {
         const DpGrid g = dp_grid(A, N);
         float* partial = static_cast<float*>(ws);

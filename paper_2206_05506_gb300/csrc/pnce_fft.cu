@@ -639,6 +639,9 @@ bool fft_applies(int N, int KL) {
 // 1.7e-7; N = 300, 75 lags 1.6e-7 / 1.7e-7, 150 lags 2.2e-7 / 1.8e-7; the pilot gradient alike.
 // (The forward sums N terms: N = 60 1.3e-7 / 0.7e-7, N = 2047 6.8e-7 / 1.1e-7.)
 bool fft_adjoint_applies(int N, int KL) { return KL >= 128 && fft_applies(N, KL); }
+// The pilot gradient sums the rows too, and the two meet earlier: N = 511, 64 lags 1.9e-7 / 1.8e-7,
+// N = 200, 50 lags 2.0e-7 / 2.3e-7, 24 lags 1.5e-7 / 2.1e-7.
+bool fft_dp_applies(int N, int KL) { return KL >= 48 && fft_applies(N, KL); }
 
 cudaError_t launch_fft_forward(const float* p, bool tanh_map, const float2* Y, long long A, int N,
                                int KL, float2* H, cudaStream_t s) {
