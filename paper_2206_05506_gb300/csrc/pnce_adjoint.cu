@@ -17,7 +17,7 @@
 // (t < 32 R + 136) and G[a][j0 .. j0+127] in its own shared buffers with cp.async,
 // double buffered so that the next item's copies fly while this one is summed.  A lane's
 // R outputs read Y at consecutive offsets: an (R + 7)-entry register window slides along
-// the staged row (fully unrolled, so the slide is only register renaming), and the real
+// the staged row (unrolled, so the slide is only register renaming), and the real
 // and imaginary products go into the two halves of packed FP32 FMAs.  Each warp writes
 // one partial row; a second kernel adds the partial rows of each q-tile in a fixed
 // order.  The result is bitwise reproducible.
@@ -36,7 +36,7 @@ struct DpShape {
     static constexpr int QT = 32 * R;             // outputs per warp tile
     static constexpr int WN = R + 7;              // register window entries
     static constexpr int WLEN = JC + QT + 8;      // staged window entries (a lane reads up to
-                                                  // R*31 + WN + 8*14 + 7 < WLEN)
+                                                  // R*31 + WN + 8*15 + 7 < WLEN)
     static constexpr int WPAD = ((WLEN + WLEN / R + 1) + 1) & ~1;   // even: g 16-byte aligned
 };
 
@@ -90,6 +90,22 @@ __device__ __forceinline__ void dp_stage(DpStage<R>& st, const float2* yrow, con
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
+// acc[r] += g[u] w[r + u] for the eight lags u = 0 .. 7, real and imaginary products apart
+template <int R>
+__device__ __forceinline__ void dp_group(float2 (&acc)[R], const float2 (&w)[DpShape<R>::WN],
+                                         const float2* g) {
+    const float4* g4 = reinterpret_cast<const float4*>(g);
+#pragma unroll
+    for (int u2 = 0; u2 < 4; ++u2) {
+        const float4 gg = g4[u2];
+        const float2 ga = make_float2(gg.x, gg.y), gb = make_float2(gg.z, gg.w);
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = __ffma2_rn(ga, w[2 * u2 + r], acc[r]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = __ffma2_rn(gb, w[2 * u2 + 1 + r], acc[r]);
+    }
+}
+
 template <int R>
 __global__ void __launch_bounds__(DP_WPB * 32, 2)
 dp_partial_kernel(const float2* __restrict__ G, const float2* __restrict__ Y, long long A, int N,
@@ -105,7 +121,7 @@ dp_partial_kernel(const float2* __restrict__ G, const float2* __restrict__ Y, lo
     // items i = a * chunks + c for i = slot, slot + P, ... < A * chunks (slot < P <= A)
     const long long items = (A * chunks - slot + P - 1) / P;
     long long next_a = slot / chunks;
-    int next_c = (int)(slot % chunks);
+    int next_c = (int)(slot % chunks), cur_c = next_c;
     const long long step_a = P / chunks;
     const int step_c = (int)(P % chunks);
     auto issue = [&](DpStage<R>& st) {
@@ -134,32 +150,46 @@ dp_partial_kernel(const float2* __restrict__ G, const float2* __restrict__ Y, lo
         const DpStage<R>& st = buf[k & 1];
         // output q0 + R*lane + r at lag j0 + u reads window entry R*lane + r + u
         const int base = R * lane;
-        float2 w[WN];
+        const int lags = KL - cur_c * JC < JC ? KL - cur_c * JC : JC;
+        cur_c += step_c;
+        if (cur_c >= chunks) cur_c -= chunks;
+        // Only the chunk's own lags are summed (a zero in the place of a lag past K*L would make a
+        // sample that is no number reach outputs that it has no part in): 96 at once where there
+        // are as many, then 16 by 16, then the rest one by one.  Against whole chunks of 128,
+        // kernel time in us: 4096 rows of N = 1023, 8 lags 60.3 -> 27.6, 40 lags 60.4 -> 35.5; 1024
+        // rows of N = 4100, 128 lags 60.3 -> 58.2, 500 lags 193 -> 183; 512 rows of N = 8191, 2048
+        // lags 660 -> 606.  (16 by 16 throughout: 500 lags 212.)
+        const float2 *wp = st.w + wpos<R>(base), *g = st.g;
+        int left = lags;
+        float2 w[WN], nw[8];
 #pragma unroll
-        for (int i = 0; i < WN; ++i) w[i] = st.w[wpos<R>(base + i)];
+        for (int i = 0; i < WN; ++i) w[i] = wp[wpos<R>(i)];
+        auto step = [&](int s) {              // lags 8 s .. 8 s + 7, and the window moves on
 #pragma unroll
-        for (int s = 0; s < JC / 8; ++s) {
-            float2 nw[8];
-            if (s + 1 < JC / 8) {
+            for (int i = 0; i < 8; ++i) nw[i] = wp[wpos<R>(8 * s + WN + i)];
+            dp_group<R>(acc, w, g + 8 * s);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) nw[i] = st.w[wpos<R>(base + 8 * s + WN + i)];
-            }
-            const float4* g4 = reinterpret_cast<const float4*>(st.g + 8 * s);
+            for (int i = 0; i < WN - 8; ++i) w[i] = w[i + 8];
 #pragma unroll
-            for (int u2 = 0; u2 < 4; ++u2) {
-                const float4 gg = g4[u2];
-                const float2 ga = make_float2(gg.x, gg.y), gb = make_float2(gg.z, gg.w);
+            for (int i = 0; i < 8; ++i) w[WN - 8 + i] = nw[i];
+        };
+        if (left >= JC - 32) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = __ffma2_rn(ga, w[2 * u2 + r], acc[r]);
+            for (int s = 0; s < JC / 8 - 4; ++s) step(s);
+            left -= JC - 32;
+            wp += wpos<R>(JC - 32);
+            g += JC - 32;
+        }
+#pragma unroll 1
+        for (; left >= 16; left -= 16, wp += wpos<R>(16), g += 16) {
+            step(0);
+            step(1);
+        }
+        if (left & 8) dp_group<R>(acc, w, g);
+        for (int u = left & 8; u < left; ++u) {
+            const float2 gu = g[u];
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = __ffma2_rn(gb, w[2 * u2 + 1 + r], acc[r]);
-            }
-            if (s + 1 < JC / 8) {
-#pragma unroll
-                for (int i = 0; i < WN - 8; ++i) w[i] = w[i + 8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) w[WN - 8 + i] = nw[i];
-            }
+            for (int r = 0; r < R; ++r) acc[r] = __ffma2_rn(gu, wp[wpos<R>(r + u)], acc[r]);
         }
         __syncwarp();                         // every lane is done with this stage
     }
