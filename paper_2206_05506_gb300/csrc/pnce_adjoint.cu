@@ -1,5 +1,6 @@
 // Adjoint of the real-pilot correlation (pilot optimisation through the estimator): the
-// entry to it, and the dense kernels for shapes beyond the transform lengths of pnce_fft.cu.
+// entry to it, and the dense kernels for the shapes that pnce_fft.cu does not take (fewer than
+// 128 lags, or transforms longer than 4096).
 //
 // Forward: H[a][j] = (1/N) sum_n Y[a][n] p[(n - j) mod N], p real.  For a real loss with
 // G = dLoss/dRe(H) + i dLoss/dIm(H):
@@ -263,7 +264,7 @@ cudaError_t launch_dp(const DpGrid& g, const float2* G, const float2* Y, long lo
 namespace pnce {
 
 size_t backward_workspace(long long A, int N, int KL) {
-    if (fft_dp_applies(N, KL)) return fft_adjoint_workspace(A, N, KL);
+    if (fft_adjoint_applies(N, KL)) return fft_adjoint_workspace(A, N, KL);
     const DpGrid g = dp_grid(A, N);
     return round_up((size_t)(g.P * g.Q) * (size_t)g.QT * sizeof(float), 256);
 }
@@ -278,8 +279,6 @@ cudaError_t launch_backward(const float* p, bool tanh_map, const float2* Y, cons
         cudaError_t e = launch_adjoint_dy(p, tanh_map, G, A, N, KL, dY, s);
         if (e != cudaSuccess) return e;
     }
-    if (dp && fft_dp_applies(N, KL))
-        return launch_fft_adjoint(p, tanh_map, G, Y, A, N, KL, nullptr, dp, ws, s);
     if (dp) {
         const DpGrid g = dp_grid(A, N);
         float* partial = static_cast<float*>(ws);

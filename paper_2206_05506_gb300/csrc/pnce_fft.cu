@@ -633,15 +633,14 @@ bool fft_applies(int N, int KL) {
     return with_length(N, KL, false, [](auto) { return true; });
 }
 
-// The adjoint sums K*L terms (dY) or rows times K*L of them: with few lags the dense kernels are
-// the more exact ones.  Relative error against 64 bits, dense / transform, 300 rows, dY: N = 1023,
-// 8 lags 5.9e-8 / 1.5e-7, 64 lags 1.5e-7 / 1.6e-7, 255 lags 2.9e-7 / 1.8e-7; N = 511, 127 lags 2.0e-7 /
-// 1.7e-7; N = 300, 75 lags 1.6e-7 / 1.7e-7, 150 lags 2.2e-7 / 1.8e-7; the pilot gradient alike.
+// The adjoint sums K*L terms (dY) or rows times K*L of them (pilot gradient): with few lags the
+// dense kernels are the more exact ones.  Relative error against 64 bits, dense / transform: dY, 300
+// rows, N = 1023, 8 lags 5.9e-8 / 1.5e-7, 64 lags 1.5e-7 / 1.6e-7, 255 lags 2.9e-7 / 1.8e-7; N = 300,
+// 75 lags 1.6e-7 / 1.7e-7, 150 lags 2.2e-7 / 1.8e-7; pilot gradient, 40 rows, N = 200, 48 lags
+// 1.5e-7 / 2.3e-7, N = 2047, 64 lags 1.7e-7 / 2.0e-7, N = 300, 96 lags 1.9e-7 / 2.1e-7; from 128 lags
+// on it is no larger by transform for any of 1 to 2048 rows, N = 128 to 2047.
 // (The forward sums N terms: N = 60 1.3e-7 / 0.7e-7, N = 2047 6.8e-7 / 1.1e-7.)
 bool fft_adjoint_applies(int N, int KL) { return KL >= 128 && fft_applies(N, KL); }
-// The pilot gradient sums the rows too, and the two meet earlier: N = 511, 64 lags 1.9e-7 / 1.8e-7,
-// N = 200, 50 lags 2.0e-7 / 2.3e-7, 24 lags 1.5e-7 / 2.1e-7.
-bool fft_dp_applies(int N, int KL) { return KL >= 48 && fft_applies(N, KL); }
 
 cudaError_t launch_fft_forward(const float* p, bool tanh_map, const float2* Y, long long A, int N,
                                int KL, float2* H, cudaStream_t s) {

@@ -1,6 +1,7 @@
 """The pilot gradient where it is delicate: samples that are not numbers, which reach exactly
 the entries whose sums they are part of, for lag counts around the kernels' steps (8 lags, a
-chunk of 128) and for pilots shorter and longer than their windows."""
+chunk of 128) and for pilots shorter and longer than their windows; and, below 128 lags, the
+dense sum's exactness."""
 import numpy as np
 import pytest
 import torch
@@ -37,3 +38,17 @@ def test_a_sample_that_is_no_number_reaches_its_own_entries(A, N, KL):
     assert np.array_equal(np.isnan(dp), hit)
     if not hit.all():
         assert O.nmse(dp[~hit], want[~hit]) <= 1e-10
+
+
+@pytest.mark.parametrize("N, KL", [(60, 48), (200, 64), (300, 100), (1023, 127), (2047, 48)])
+def test_few_lags_are_summed_directly(N, KL):
+    # one gradient that is not zero and whole-numbered samples: every entry is one product, so
+    # it is exact but for 1/N and the product with it, 2^-24 each, and zero where the sample is
+    rng = np.random.default_rng([N, KL])
+    A, a, j = 3, 1, KL - 2
+    Y = (rng.integers(-4, 5, (1, A, N)) + 1j * rng.integers(-4, 5, (1, A, N))).astype(np.complex64)
+    G = np.zeros((1, A, 1, KL), dtype=np.complex64)
+    G[0, a, 0, j] = 1
+    dp = _dp(rng.standard_normal(N).astype(np.float32), Y, G, KL).astype(np.float64)
+    want = np.roll(Y[0, a].real.astype(np.float64), -j) / N
+    assert np.all(np.abs(dp - want) <= 2.0 ** -23 * np.abs(want))
