@@ -200,8 +200,8 @@ typedef enum {
 
 /*
  * Estimate with a real-valued pilot (float32 [N], device) in place of the +-1 sequence:
- * H = (1/N) sum_n Y[n] p[(n - j) mod N], FP32 on the CUDA cores (by FFT up to N + K*L - 1 =
- * 4096; rows that hold or reach infinities are summed directly).  With PNCE_PILOT_TANH
+ * H = (1/N) sum_n Y[n] p[(n - j) mod N], FP32 on the CUDA cores (by FFT for N >= 84 up to
+ * N + K*L - 1 = 4096; rows that hold or reach infinities are summed directly).  With PNCE_PILOT_TANH
  * the argument is theta and p = tanh(theta) is formed inside the kernel: the forward of
  * the relaxed pilot used for end-to-end pilot optimisation.
  */

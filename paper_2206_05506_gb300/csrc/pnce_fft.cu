@@ -24,7 +24,8 @@
 // share the transform of G); 2048 rows of N = 2047, 300 lags: 189 -> 46, 116 -> 48, 137 -> 43
 // us; even with 1-8 lags, where the dense kernel still pays for a tile of 256, N = 1023: 97 ->
 // 42 us.  Error against 64 bits, N = 1023: 5e-7 -> 2e-7 (fewer roundings per output).  Lengths
-// above 4096 (N + K*L - 1) stay with the dense kernels.
+// above 4096 (N + K*L - 1) stay with the dense kernels, and so do the shapes where these are the
+// more exact ones (fft_forward_applies, fft_adjoint_applies).
 //
 // A row whose values are not numbers, or so large that an intermediate overflows, comes out
 // of the transforms as infinities and NaN throughout; every such output is summed again
@@ -35,7 +36,8 @@
 
 namespace {
 
-constexpr int MIN_LOG = 6, MAX_LOG = 12;       // transform lengths 64 .. 4096
+constexpr int MIN_LOG = 7, MAX_LOG = 12;       // transform lengths 128 .. 4096
+constexpr int MIN_ADJOINT_LOG = 8;             // of the adjoint (128 lags and more)
 
 template <int LS>
 struct Fft {
@@ -608,14 +610,16 @@ struct Launch {
     }
 };
 
-// Calls f(Launch<LS>) for the transform length of the shape; def where there is none.
-template <class Fn, class T>
+// Calls f(Launch<LS>) for the transform length of the shape, 2^MIN at least; def where there is
+// none.
+template <int MIN, class Fn, class T>
 T with_length(int N, int KL, T def, Fn f) {
-    int ls = MIN_LOG;
+    int ls = MIN;
     while (ls <= MAX_LOG && (1 << ls) < N + KL - 1) ++ls;
+    if constexpr (MIN <= 7) {
+        if (ls == 7) return f(Launch<7>());
+    }
     switch (ls) {
-        case 6: return f(Launch<6>());
-        case 7: return f(Launch<7>());
         case 8: return f(Launch<8>());
         case 9: return f(Launch<9>());
         case 10: return f(Launch<10>());
@@ -629,9 +633,12 @@ T with_length(int N, int KL, T def, Fn f) {
 
 namespace pnce {
 
-bool fft_applies(int N, int KL) {
-    return with_length(N, KL, false, [](auto) { return true; });
-}
+static bool fft_applies(int N, int KL) { return N + KL - 1 <= 1 << MAX_LOG; }
+
+// The forward sums N terms, and for short pilots the dense sum of them is the more exact one.
+// Error against 64 bits, transform over dense, 400 rows, at the lag count where it is largest: N = 31
+// 1.5, N = 62 1.18, N = 64 1.06, N = 71 1.07, N = 83 1.04; N = 84 .. 130 0.77 .. 0.99, N = 2047 0.16.
+bool fft_forward_applies(int N, int KL) { return N >= 84 && fft_applies(N, KL); }
 
 // The adjoint sums K*L terms (dY) or rows times K*L of them (pilot gradient): with few lags the
 // dense kernels are the more exact ones.  Relative error against 64 bits, dense / transform: dY, 300
@@ -639,26 +646,25 @@ bool fft_applies(int N, int KL) {
 // 75 lags 1.6e-7 / 1.7e-7, 150 lags 2.2e-7 / 1.8e-7; pilot gradient, 40 rows, N = 200, 48 lags
 // 1.5e-7 / 2.3e-7, N = 2047, 64 lags 1.7e-7 / 2.0e-7, N = 300, 96 lags 1.9e-7 / 2.1e-7; from 128 lags
 // on it is no larger by transform for any of 1 to 2048 rows, N = 128 to 2047.
-// (The forward sums N terms: N = 60 1.3e-7 / 0.7e-7, N = 2047 6.8e-7 / 1.1e-7.)
 bool fft_adjoint_applies(int N, int KL) { return KL >= 128 && fft_applies(N, KL); }
 
 cudaError_t launch_fft_forward(const float* p, bool tanh_map, const float2* Y, long long A, int N,
                                int KL, float2* H, cudaStream_t s) {
     if (A <= 0) return cudaSuccess;
-    return with_length(N, KL, cudaErrorNotSupported, [&](auto l) {
+    return with_length<MIN_LOG>(N, KL, cudaErrorNotSupported, [&](auto l) {
         return l.forward(p, tanh_map, Y, A, N, KL, H, s);
     });
 }
 
 size_t fft_adjoint_workspace(long long A, int N, int KL) {
-    return with_length(N, KL, (size_t)0, [&](auto l) { return l.workspace(A); });
+    return with_length<MIN_ADJOINT_LOG>(N, KL, (size_t)0, [&](auto l) { return l.workspace(A); });
 }
 
 cudaError_t launch_fft_adjoint(const float* p, bool tanh_map, const float2* G, const float2* Y,
                                long long A, int N, int KL, float2* dY, float* dp, void* ws,
                                cudaStream_t s) {
     if (A <= 0 || (!dY && !dp)) return cudaSuccess;
-    return with_length(N, KL, cudaErrorNotSupported, [&](auto l) {
+    return with_length<MIN_ADJOINT_LOG>(N, KL, cudaErrorNotSupported, [&](auto l) {
         return l.adjoint(p, tanh_map, G, Y, A, N, KL, dY, dp, ws, s);
     });
 }

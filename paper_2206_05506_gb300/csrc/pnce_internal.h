@@ -221,7 +221,7 @@ size_t backward_workspace(long long A, int N, int KL);
 // Real-valued pilots by FFT (pnce_fft.cu), for shapes whose transform length is at most 4096:
 // forward, and the adjoint (dY and dp either may be null; ws: fft_adjoint_workspace bytes, for
 // dp only).
-bool fft_applies(int N, int KL);
+bool fft_forward_applies(int N, int KL);
 bool fft_adjoint_applies(int N, int KL);
 cudaError_t launch_fft_forward(const float* p, bool tanh_map, const float2* Y, long long A, int N,
                                int KL, float2* H, cudaStream_t s);

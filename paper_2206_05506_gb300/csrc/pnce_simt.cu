@@ -684,7 +684,7 @@ cudaError_t launch_simt_bits_ex(const pnce_pilot* pilot, const float2* Y, long l
 
 cudaError_t launch_simt_real(const float* p, bool tanh_map, const float2* Y, long long A, int N,
                              int KL, float2* H, cudaStream_t s) {
-    if (fft_applies(N, KL)) return launch_fft_forward(p, tanh_map, Y, A, N, KL, H, s);
+    if (fft_forward_applies(N, KL)) return launch_fft_forward(p, tanh_map, Y, A, N, KL, H, s);
     const LagMap lm = lagmap_contiguous(KL);
     return tanh_map ? launch<FWD_TANH>(nullptr, p, Y, N, A, N, lm, N, H, s)
                     : launch<FWD_REAL>(nullptr, p, Y, N, A, N, lm, N, H, s);
