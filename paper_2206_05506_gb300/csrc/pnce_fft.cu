@@ -29,7 +29,7 @@
 //
 // A row whose values are not numbers, or so large that an intermediate overflows, comes out
 // of the transforms as infinities and NaN throughout; every such output is summed again
-// directly, in the order of the dense kernel.
+// directly, in the order of the dense kernel (the pilot gradient: direct_dp).
 #include <algorithm>
 
 #include "pnce_internal.h"
@@ -52,7 +52,11 @@ struct Fft {
     static constexpr int X1 = 16 * LD1;                      // first exchange, entries
     static constexpr int LD2 = 16 * (M2 + 1) + M2;
     static constexpr int X2 = M2 > 1 ? 16 * LD2 : 0;         // second exchange, same buffer
-    static constexpr int ROW = X1 > X2 ? X1 : X2;
+    // direct_sums: one entry of padding per 16, and 16 outputs past the last one (the longer
+    // transforms' exchanges have the room)
+    static constexpr int XD = LS == 8 ? S + S / 16 + 32 : 0;
+    static constexpr int ROW = X1 > X2 ? (X1 > XD ? X1 : XD) : X2 > XD ? X2 : XD;
+    static_assert(LS < 8 || ROW >= S + S / 16 + 32, "direct_sums");
     static constexpr int TW2 = M2 > 1 ? 15 * M2 : 0;         // second twiddles, [k - 1][m2]
     // entries of dynamic shared memory: a spectrum, the second twiddles, the rows' buffers
     static constexpr int SMEM = S + (TW2 + 1) / 2 * 2 + RT * ROW;
@@ -391,6 +395,64 @@ fft_forward_kernel(const float* __restrict__ p, bool tanh_map, const float2* __r
     }
 }
 
+// acc[r] += in[k] e[16 t + r + k] for k = 0, 1, .. in order (real parts and imaginary parts apart),
+// with e[q] at x[q + q / 16]: 16 consecutive outputs per thread, so that a step of one k takes one
+// new entry of e, its 8-byte loads free of bank conflicts.
+__device__ __forceinline__ void direct_sums(float2 (&acc)[16], const float2* x, const float2* in,
+                                            int in_len, int t) {
+    const float2* e = x + 17 * t;
+    float2 w[31];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) w[i] = e[i];
+    int k = 0;
+#pragma unroll 1
+    for (; k + 16 <= in_len; k += 16, e += 17, in += 16) {
+        w[15] = e[15];
+#pragma unroll
+        for (int i = 16; i < 31; ++i) w[i] = e[i + 1];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const float2 v = __ldg(in + u);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) acc[r] = __ffma2_rn(v, w[r + u], acc[r]);
+        }
+#pragma unroll
+        for (int i = 0; i < 15; ++i) w[i] = w[i + 16];
+    }
+    for (int u = 0; k < in_len; ++k, ++u) {
+        const float2 v = __ldg(in + u);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) acc[r] = __ffma2_rn(v, e[r + u + (r + u) / 16], acc[r]);
+    }
+}
+
+// The pilot gradient's sums of the rows row0, row0 + stride, .. (row0 = first + sub) formed
+// directly, in order: slot[i] = (NaN, r[i] + r[i - N]) for i < N, (NaN, 0) above.  In place of a
+// spectrum that is not finite: the NaN marks the slot, and fft_dp_final_kernel adds the sums.  Every block does this
+// for its own rows, so that such a row costs its block's rows a direct sum and no more.  Pilot
+// gradient of 4096 rows of N = 1023, 512 lags, us: 38.8; a NaN in one row 179, in every row 293 (the
+// dense kernel 182; every entry summed by itself in fft_dp_final_kernel: 146000).
+template <int LS>
+__device__ __noinline__ void direct_dp(const float2* G, const float2* Y, long long first, int sub,
+                                       long long stride, long long A, int N, int KL, int t,
+                                       float2* x, float2* slot) {
+    float2 acc[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) acc[r] = make_float2(0.f, 0.f);
+    for (; first < A; first += stride) {
+        const long long row = first + sub;
+        if (row < A) {
+            const float2* y = Y + row * N;
+            for (int q = t; q < N + KL - 1; q += Fft<LS>::M) x[q + q / 16] = __ldg(y + (q < N ? q : q - N));
+        }
+        row_sync<Fft<LS>::M>();
+        if (row < A && 16 * t < N) direct_sums(acc, x, G + row * KL, KL, t);
+        row_sync<Fft<LS>::M>();
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) slot[16 * t + r] = make_float2(nanf(""), acc[r].x + acc[r].y);
+}
+
 // Adjoint.  Block b takes the rows b, b + blocks, .. in order; per row the spectrum of G gives
 // dY (times the pilot's) and, times the conjugate, meets that of Y: DP adds these products
 // over the block's rows and stores the sum, [k][t].  The number of blocks depends on the
@@ -436,44 +498,67 @@ fft_adjoint_kernel(const float* __restrict__ p, bool tanh_map, const float2* __r
     }
     if constexpr (DP) {
         float2* o = partial + ((long long)blockIdx.x * F::RT + sub) * F::S;
+        bool fine = true;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) o[k * F::M + t] = acc[k];
+        for (int k = 0; k < 16; ++k) {
+            fine = fine && fmaf(0.f, acc[k].x, 0.f * acc[k].y) == 0.f;
+            o[k * F::M + t] = acc[k];
+        }
+        if (__syncthreads_or(!fine))
+            direct_dp<LS>(G, Y, (long long)blockIdx.x * F::RT, sub, (long long)gridDim.x * F::RT, A,
+                          N, KL, t, team.x, o);
     }
 }
 
+// A slot of direct sums (direct_dp) counts as zero among the spectra.
+__device__ __forceinline__ float2 spectrum_of(float2 q) {
+    return isnan(q.x) ? make_float2(0.f, 0.f) : q;
+}
+
 // spec[i] = sum over the P partial spectra, in a fixed order: warp w of a block adds
-// w, w + 32, .. for 32 consecutive i, then the 32 sums in order.  A programmatic dependent
-// (partial is not declared restrict: its loads must stay behind the wait).
+// w, w + 32, .. for 32 consecutive i, then the 32 sums in order.  *direct: whether slots hold
+// direct sums.  A programmatic dependent (partial is not declared restrict: its loads must stay
+// behind the wait).
 __global__ void __launch_bounds__(1024)
-fft_dp_sum_kernel(const float2* partial, int P, int S, float2* spec) {
+fft_dp_sum_kernel(const float2* partial, int P, int S, float2* spec, int* direct) {
     __shared__ float2 red[32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float2 s = make_float2(0.f, 0.f);
+    bool any = false;
 #pragma unroll 8
     for (int b = warp; b < P; b += 32) s = cadd(s, partial[(long long)b * S + i]);
+    if (isnan(s.x)) {                          // slots of direct sums: once more without them
+        s = make_float2(0.f, 0.f);
+        for (int b = warp; b < P; b += 32) {
+            const float2 q = partial[(long long)b * S + i];
+            any |= isnan(q.x);
+            s = cadd(s, spectrum_of(q));
+        }
+    }
     red[warp][lane] = s;
-    __syncthreads();
+    any = __syncthreads_or(any);
     if (warp == 0) {
         float2 r = make_float2(0.f, 0.f);
 #pragma unroll
         for (int w = 0; w < 32; ++w) r = cadd(r, red[w][lane]);
         spec[i] = r;
+        if (i == 0) *direct = any;
     }
 }
 
 // Every block: r = IFFT(spec), then for its 32 consecutive i, dp[i] = (1/N) Re(r[i] + r[i - N])
-// (times 1 - tanh(theta)^2).  A result that is not finite is summed again directly by the
-// whole block, its threads in a fixed pattern.  A programmatic dependent.
+// (times 1 - tanh(theta)^2), plus the direct sums where there are any.  Where that is not finite,
+// the sum of the spectra or its transform may have overflowed: the block then adds the spectra
+// again scaled by 2^-20 (slots times S is less, so that no sum can overflow) and transforms that.
+// A programmatic dependent.
 template <int LS>
 __global__ void __launch_bounds__(Fft<LS>::THREADS)
-fft_dp_final_kernel(const float2* spec, const float2* __restrict__ G,
-                    const float2* __restrict__ Y, long long A, int N, int KL,
-                    const float* __restrict__ theta, float* __restrict__ dp) {
+fft_dp_final_kernel(const float2* spec, const float2* partial, int P, const int* direct, int N,
+                    int KL, const float* __restrict__ theta, float* __restrict__ dp) {
     using F = Fft<LS>;
     extern __shared__ __align__(16) float2 fft_smem[];
-    __shared__ unsigned bad;
     __shared__ float red[F::THREADS];
     float* r = reinterpret_cast<float*>(fft_smem);
     float2* tw2 = fft_smem + F::S;
@@ -485,46 +570,60 @@ fft_dp_final_kernel(const float2* spec, const float2* __restrict__ G,
     float2 v[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = spec[k * F::M + t];
+    const bool any = *direct != 0;
     team.inverse(v);
     if (sub == 0) {
 #pragma unroll
         for (int k = 0; k < 16; ++k) r[k * F::M + t] = v[k].x;
     }
-    __syncthreads();
-    const int i0 = blockIdx.x * 32;
-    float deriv = 1.f;
-    if (threadIdx.x < 32) {
-        const int i = i0 + threadIdx.x;
-        float s = 0.f;
-        if (i < N) {
-            if (theta) {
-                const float th = tanhf(theta[i]);
-                deriv = 1.0f - th * th;
-            }
-            s = (i > N - KL ? r[i] + r[F::S + i - N] : r[i]) * (1.0f / ((float)N * (float)F::S));
-            dp[i] = s * deriv;
-        }
-        const unsigned b = __ballot_sync(0xffffffffu, !isfinite(s));
-        if (threadIdx.x == 0) bad = b;
-    }
-    __syncthreads();
-    for (unsigned b = bad; b; b &= b - 1) {
-        const int i = i0 + __ffs(b) - 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    if (any) {
         float x = 0.f;
-        for (long long e = threadIdx.x; e < A * KL; e += F::THREADS) {
-            const long long a = e / KL;
-            const int j = (int)(e - a * KL);
-            const float2 g = G[e], y = Y[a * N + (i + j < N ? i + j : i + j - N)];
-            x = fmaf(g.x, y.x, fmaf(g.y, y.y, x));
+        if (i < N) {
+#pragma unroll 4
+            for (int b = warp; b < P; b += F::THREADS / 32) {
+                const float2 q = partial[(long long)b * F::S + i];
+                x += isnan(q.x) ? q.y : 0.f;
+            }
         }
         red[threadIdx.x] = x;
-        __syncthreads();
-        if (threadIdx.x == (unsigned)(i - i0)) {
-            x = 0.f;
-            for (int w = 0; w < F::THREADS; ++w) x += red[w];
-            dp[i] = x * (1.0f / (float)N) * deriv;
+    }
+    __syncthreads();
+    const float scale = 1.0f / ((float)N * (float)F::S);
+    float deriv = 1.f, s = 0.f, x = 0.f;
+    if (warp == 0 && i < N) {
+        if (theta) {
+            const float th = tanhf(theta[i]);
+            deriv = 1.0f - th * th;
+        }
+        s = (i > N - KL ? r[i] + r[F::S + i - N] : r[i]) * scale;
+        if (any) {
+            for (int w = 0; w < F::THREADS / 32; ++w) x += red[32 * w + lane];
+            x *= 1.0f / (float)N;
+        }
+        dp[i] = (s + x) * deriv;
+    }
+    if (!__syncthreads_or(!isfinite(s))) return;
+    const float down = 0x1p-20f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        v[k] = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int b = sub; b < P; b += F::RT)
+            v[k] = __ffma2_rn(spectrum_of(partial[(long long)b * F::S + k * F::M + t]),
+                              make_float2(down, down), v[k]);
+    }
+    team.inverse(v);
+    for (int w = 0; w < F::RT; ++w) {
+        if (sub == w) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[k * F::M + t] = (w ? r[k * F::M + t] : 0.f) + v[k].x;
         }
         __syncthreads();
+    }
+    if (warp == 0 && i < N && !isfinite(s)) {
+        s = (i > N - KL ? r[i] + r[F::S + i - N] : r[i]) * (scale / down);
+        dp[i] = (s + x) * deriv;
     }
 }
 
@@ -585,7 +684,8 @@ struct Launch {
     }
 
     static size_t workspace(long long A) {
-        return sizeof(float2) * (size_t)F::S * ((size_t)adjoint_blocks(A, true) * F::RT + 1);
+        // the sum, the partial spectra, fft_dp_sum_kernel's flag
+        return sizeof(float2) * ((size_t)F::S * ((size_t)adjoint_blocks(A, true) * F::RT + 1) + 1);
     }
 
     static cudaError_t adjoint(const float* p, bool tanh_map, const float2* G, const float2* Y,
@@ -599,13 +699,15 @@ struct Launch {
         kern<<<blocks, F::THREADS, smem, s>>>(p, tanh_map, G, Y, A, N, KL, dY,
                                               dp ? spec + F::S : nullptr);
         if ((e = cudaGetLastError()) != cudaSuccess || !dp) return e;
-        if ((e = launch_dependent(fft_dp_sum_kernel, F::S / 32, 1024, 0, s,
-                                  (const float2*)(spec + F::S), blocks * F::RT, F::S, spec)) !=
-            cudaSuccess)
+        const int slots = blocks * F::RT;
+        const float2* partial = spec + F::S;
+        int* direct = reinterpret_cast<int*>(spec + (size_t)F::S * (slots + 1));
+        if ((e = launch_dependent(fft_dp_sum_kernel, F::S / 32, 1024, 0, s, partial, slots, F::S,
+                                  spec, direct)) != cudaSuccess)
             return e;
         if ((e = limit(fft_dp_final_kernel<LS>)) != cudaSuccess) return e;
         return launch_dependent(fft_dp_final_kernel<LS>, (unsigned)((N + 31) / 32), F::THREADS, smem,
-                                s, (const float2*)spec, G, Y, A, N, KL,
+                                s, (const float2*)spec, partial, slots, (const int*)direct, N, KL,
                                 tanh_map ? p : (const float*)nullptr, dp);
     }
 };

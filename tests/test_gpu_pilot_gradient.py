@@ -52,3 +52,74 @@ def test_few_lags_are_summed_directly(N, KL):
     dp = _dp(rng.standard_normal(N).astype(np.float32), Y, G, KL).astype(np.float64)
     want = np.roll(Y[0, a].real.astype(np.float64), -j) / N
     assert np.all(np.abs(dp - want) <= 2.0 ** -23 * np.abs(want))
+
+
+def _median_ms(f, n=5):
+    f()
+    out = []
+    for _ in range(n):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        b.synchronize()
+        out.append(a.elapsed_time(b))
+    return sorted(out)[n // 2]
+
+
+@pytest.mark.parametrize("A, N, KL", [(1, 128, 128), (7, 129, 128), (3000, 200, 130), (2500, 1023, 256),
+                                      (700, 2047, 512)])
+def test_values_that_are_not_finite_by_transform(A, N, KL):
+    # A row whose transform overflows while its products do not; a sample that is no number;
+    # infinities; a gradient that is no number.  The entries that these reach are what the
+    # direct sum gives, the others are the oracle's (tolerance as in test_gpu_fft), and none of
+    # it costs more than the direct sums of the blocks concerned: 2 A N K L operations, far
+    # below a hundred times the transforms' time.
+    import paper_2206_05506_gb300 as pk
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator(dev).manual_seed(N)
+    Y = torch.randn(1, A, N, dtype=torch.complex64, device=dev, generator=gen)
+    G = torch.randn(1, A, 1, KL, dtype=torch.complex64, device=dev, generator=gen)
+    p = torch.randn(N, device=dev, generator=gen)
+
+    def dp(Y, G):
+        return pk.backward(p, Y, G, 1, KL, need_dY=False)[1]
+
+    def want(Y, G):
+        Gf = torch.zeros(A, N, dtype=torch.complex128, device=dev)
+        Gf[:, :KL] = G[0, :, 0]
+        cross = (torch.fft.fft(Gf).conj() * torch.fft.fft(Y[0].to(torch.complex128))).sum(0)
+        return torch.fft.ifft(cross).real / N
+
+    def close(a, b):
+        return float(torch.linalg.norm(a - b) / torch.linalg.norm(b)) ** 2 <= 1e-11
+
+    n, at, a = torch.arange(N, device=dev), N // 3, A - 1
+    hit = torch.isin(n, (at - torch.arange(KL, device=dev)) % N)
+    clean = want(Y, G)
+    t0 = _median_ms(lambda: dp(Y, G))
+    # overflow of the transform alone: partial sums of up to K L numbers near 3e38 / 8
+    big, small = G.clone(), Y.clone()
+    big[0, a] *= 4e37
+    small[0, a] *= 1e-30
+    assert close(dp(small, big), want(small, big))
+    # one sample that is no number, one that is infinite
+    for v in (complex(0, float("nan")), complex(float("inf"), 0)):
+        odd = Y.clone()
+        odd[0, a, at] = v
+        got = dp(odd, G)
+        assert torch.equal(torch.isfinite(got), ~hit)
+        assert torch.equal(torch.isnan(got), hit & bool(np.isnan(v.imag)))
+        if v.real:
+            j = (at - n[hit]) % N
+            assert torch.equal(torch.sign(got[hit]), torch.sign(G[0, a, 0, j].real))
+        odd[0, a, at] = 0
+        if not bool(hit.all()):
+            assert close(got[~hit], want(odd, G)[~hit])
+    # gradients that are no numbers, in one row and in all of them
+    for rows in (slice(a, A), slice(0, A)):
+        odd = G.clone()
+        odd[0, rows, 0, 1] = complex(float("nan"), 0)
+        assert bool(torch.isnan(dp(Y, odd)).all())
+        assert _median_ms(lambda: dp(Y, odd)) <= 100 * t0
+    assert close(dp(Y, G), clean)                # nothing is left behind in the workspace
