@@ -52,11 +52,9 @@ struct Fft {
     static constexpr int X1 = 16 * LD1;                      // first exchange, entries
     static constexpr int LD2 = 16 * (M2 + 1) + M2;
     static constexpr int X2 = M2 > 1 ? 16 * LD2 : 0;         // second exchange, same buffer
-    // direct_sums: one entry of padding per 16, and 16 outputs past the last one (the longer
-    // transforms' exchanges have the room)
-    static constexpr int XD = LS == 8 ? S + S / 16 + 32 : 0;
-    static constexpr int ROW = X1 > X2 ? (X1 > XD ? X1 : XD) : X2 > XD ? X2 : XD;
-    static_assert(LS < 8 || ROW >= S + S / 16 + 32, "direct_sums");
+    // direct_sums: one entry of padding per 16, and 16 outputs past the last one
+    static constexpr int XD = S + S / 16 + 32;
+    static constexpr int ROW = std::max(std::max(X1, X2), XD);
     static constexpr int TW2 = M2 > 1 ? 15 * M2 : 0;         // second twiddles, [k - 1][m2]
     // entries of dynamic shared memory: a spectrum, the second twiddles, the rows' buffers
     static constexpr int SMEM = S + (TW2 + 1) / 2 * 2 + RT * ROW;
@@ -84,6 +82,15 @@ template <bool CONJ>
 __device__ __forceinline__ float2 cmul(float2 a, float2 w) {
     const float s = CONJ ? -w.y : w.y;
     return make_float2(fmaf(a.x, w.x, -a.y * s), fmaf(a.x, s, a.y * w.x));
+}
+
+// whether bad is true in any of the row's threads (M <= 32: of its warp's)
+template <int M>
+__device__ __forceinline__ bool row_any(bool bad) {
+    if constexpr (M <= 32)
+        return __any_sync(0xffffffffu, bad);
+    else
+        return __syncthreads_or(bad);
 }
 
 // DFT of length 2, 4, 8, 16 on v[B], v[B + D], ..; results in order.  INV: exponent +.
@@ -306,24 +313,6 @@ __device__ __forceinline__ float pilot_at(const float* p, bool tanh_map, int i) 
     return tanh_map ? tanhf(v) : v;
 }
 
-// out[o] = scale sum_{k < in_len} in[k] pilot[(k - o) mod N] (ADJ: pilot[(o - k) mod N]), the
-// products summed in order as the dense kernel does
-template <bool ADJ>
-__device__ __noinline__ float2 direct_sum(const float2* in, int in_len, const float* p,
-                                          bool tanh_map, int N, int o, float scale) {
-    float2 acc = make_float2(0.f, 0.f);
-    int q = ADJ ? o : (o == 0 ? 0 : N - o);
-    for (int k = 0; k < in_len; ++k) {
-        const float w = pilot_at(p, tanh_map, q);
-        const float2 y = in[k];
-        acc = make_float2(fmaf(w, y.x, acc.x), fmaf(w, y.y, acc.y));
-        q += ADJ ? -1 : 1;
-        if (q == N) q = 0;
-        if (q < 0) q = N - 1;
-    }
-    return make_float2(acc.x * scale, acc.y * scale);
-}
-
 // The pilot's spectrum of the block, [k][t]; ends with the block synchronised.
 template <int LS>
 __device__ __forceinline__ void pilot_spectrum(Team<LS>& team, const float* p, bool tanh_map, int N,
@@ -342,57 +331,6 @@ __device__ __forceinline__ void pilot_spectrum(Team<LS>& team, const float* p, b
         for (int k = 0; k < 16; ++k) Q[k * F::M + team.t] = v[k];
     }
     __syncthreads();
-}
-
-// out[o] = v scale for o < out_len; sums that are not finite are formed again directly
-template <int LS, bool ADJ>
-__device__ __forceinline__ void store_row(float2 (&v)[16], float2* out, int out_len, int t,
-                                          const float2* in, int in_len, const float* p,
-                                          bool tanh_map, int N) {
-    using F = Fft<LS>;
-    const float scale = 1.0f / ((float)N * (float)F::S);
-    bool fine = true;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int o = k * F::M + t;
-        if (o < out_len) {
-            const float2 w = make_float2(v[k].x * scale, v[k].y * scale);
-            // 0 x is 0 for finite x, NaN otherwise
-            fine = fine && fmaf(0.f, w.x, 0.f * w.y) == 0.f;
-            out[o] = w;
-        }
-    }
-    if (!fine)
-        for (int o = t; o < out_len; o += F::M)
-            if (!(isfinite(out[o].x) && isfinite(out[o].y)))
-                out[o] = direct_sum<ADJ>(in, in_len, p, tanh_map, N, o, 1.0f / (float)N);
-}
-
-// Forward: A rows Y of N samples -> KL lags.  HALF: N <= S / 2.
-template <int LS, bool HALF>
-__global__ void __launch_bounds__(Fft<LS>::THREADS, Fft<LS>::BPS)
-fft_forward_kernel(const float* __restrict__ p, bool tanh_map, const float2* __restrict__ Y,
-                   long long A, int N, int KL, float2* __restrict__ H) {
-    using F = Fft<LS>;
-    extern __shared__ __align__(16) float2 fft_smem[];
-    float2 *Q = fft_smem, *tw2 = Q + F::S;
-    const int sub = threadIdx.x / F::M, t = threadIdx.x % F::M;
-    fill_tw2<LS>(tw2);
-    Team<LS> team(fft_smem + F::SMEM - (F::RT - sub) * F::ROW, tw2, t);
-    __syncthreads();
-    pilot_spectrum<LS>(team, p, tanh_map, N, KL, sub, Q);
-    for (long long r0 = (long long)blockIdx.x * F::RT; r0 < A; r0 += (long long)gridDim.x * F::RT) {
-        const long long row = r0 + sub;
-        const bool live = row < A;
-        const float2* y = Y + row * N;
-        float2 v[16];
-        load_row<LS, HALF>(v, y, live ? N : 0, t);
-        team.template forward<HALF>(v);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = cmul<true>(v[k], Q[k * F::M + t]);
-        team.inverse(v);
-        if (live) store_row<LS, false>(v, H + row * KL, KL, t, y, N, p, tanh_map, N);
-    }
 }
 
 // acc[r] += in[k] e[16 t + r + k] for k = 0, 1, .. in order (real parts and imaginary parts apart),
@@ -424,6 +362,98 @@ __device__ __forceinline__ void direct_sums(float2 (&acc)[16], const float2* x, 
 #pragma unroll
         for (int r = 0; r < 16; ++r) acc[r] = __ffma2_rn(v, e[r + u + (r + u) / 16], acc[r]);
     }
+}
+
+// The block's rows once more, after it has stored them all: out[o] = (1/N) sum_{k < in_len} in[k]
+// pilot[(k - o) mod N] (ADJ: pilot[(o - k) mod N]) for the outputs that are not finite, the products
+// summed in order as the dense kernel does.  Behind the loop over the rows, so that it costs that
+// loop no registers and no barrier.  4096 rows of N = 1023, 512 lags, a NaN in every row, us:
+// forward 352 (43 without; the dense kernel 152), dY 272 (45; 154); one output per thread and pass,
+// as it was before, 2530 and 2984.
+template <int LS, bool ADJ>
+__device__ __noinline__ void direct_rows(float2* x, const float2* in, int in_len, float2* out,
+                                         int out_len, long long A, const float* p, bool tanh_map,
+                                         int N, int sub, int t) {
+    using F = Fft<LS>;
+    const float invN = 1.0f / (float)N;
+    for (long long first = (long long)blockIdx.x * F::RT; first < A;
+         first += (long long)gridDim.x * F::RT) {
+        const bool live = first + sub < A;
+        const long long row = live ? first + sub : first;
+        float2* const o_row = out + row * out_len;
+        bool bad = false;
+        for (int o = t; live && o < out_len; o += F::M)
+            bad |= !(isfinite(o_row[o].x) && isfinite(o_row[o].y));
+        if (!row_any<F::M>(bad)) continue;
+        // output out_len - 1 - i takes the pilot's sample for k at e[i + k]
+        for (int q = t; q < in_len + out_len - 1; q += F::M) {
+            const int m = ADJ ? N - 1 - q : q - (out_len - 1);
+            const float w = pilot_at(p, tanh_map, m < 0 ? m + N : m);
+            x[q + q / 16] = make_float2(w, w);
+        }
+        row_sync<F::M>();
+        if (live && 16 * t < out_len) {
+            float2 acc[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) acc[r] = make_float2(0.f, 0.f);
+            direct_sums(acc, x, in + row * in_len, in_len, t);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int o = out_len - 1 - 16 * t - r;
+                if (o >= 0 && !(isfinite(o_row[o].x) && isfinite(o_row[o].y)))
+                    o_row[o] = make_float2(acc[r].x * invN, acc[r].y * invN);
+            }
+        }
+        row_sync<F::M>();
+    }
+}
+
+// out[o] = v scale for o < out_len; whether all of them are finite
+template <int LS>
+__device__ __forceinline__ bool store_row(float2 (&v)[16], float2* out, int out_len, int t, int N) {
+    using F = Fft<LS>;
+    const float scale = 1.0f / ((float)N * (float)F::S);
+    bool fine = true;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int o = k * F::M + t;
+        if (o < out_len) {
+            const float2 w = make_float2(v[k].x * scale, v[k].y * scale);
+            // 0 x is 0 for finite x, NaN otherwise
+            fine = fine && fmaf(0.f, w.x, 0.f * w.y) == 0.f;
+            out[o] = w;
+        }
+    }
+    return fine;
+}
+
+// Forward: A rows Y of N samples -> KL lags.  HALF: N <= S / 2.
+template <int LS, bool HALF>
+__global__ void __launch_bounds__(Fft<LS>::THREADS, Fft<LS>::BPS)
+fft_forward_kernel(const float* __restrict__ p, bool tanh_map, const float2* __restrict__ Y,
+                   long long A, int N, int KL, float2* __restrict__ H) {
+    using F = Fft<LS>;
+    extern __shared__ __align__(16) float2 fft_smem[];
+    float2 *Q = fft_smem, *tw2 = Q + F::S;
+    const int sub = threadIdx.x / F::M, t = threadIdx.x % F::M;
+    fill_tw2<LS>(tw2);
+    Team<LS> team(fft_smem + F::SMEM - (F::RT - sub) * F::ROW, tw2, t);
+    __syncthreads();
+    pilot_spectrum<LS>(team, p, tanh_map, N, KL, sub, Q);
+    bool fine = true;
+    for (long long r0 = (long long)blockIdx.x * F::RT; r0 < A; r0 += (long long)gridDim.x * F::RT) {
+        const long long row = r0 + sub;
+        const bool live = row < A;
+        float2 v[16];
+        load_row<LS, HALF>(v, Y + row * N, live ? N : 0, t);
+        team.template forward<HALF>(v);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = cmul<true>(v[k], Q[k * F::M + t]);
+        team.inverse(v);
+        fine &= store_row<LS>(v, H + row * KL, live ? KL : 0, t, N);
+    }
+    if (__syncthreads_or(!fine))
+        direct_rows<LS, false>(team.x, Y, N, H, KL, A, p, tanh_map, N, sub, t);
 }
 
 // The pilot gradient's sums of the rows row0, row0 + stride, .. (row0 = first + sub) formed
@@ -473,18 +503,18 @@ fft_adjoint_kernel(const float* __restrict__ p, bool tanh_map, const float2* __r
     float2 acc[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) acc[k] = make_float2(0.f, 0.f);
+    bool y_fine = true;
     for (long long r0 = (long long)blockIdx.x * F::RT; r0 < A; r0 += (long long)gridDim.x * F::RT) {
         const long long row = r0 + sub;
         const bool live = row < A;
-        const float2* grow = G + row * KL;
         float2 g[16], v[16];
-        load_row<LS, true>(g, grow, live ? KL : 0, t);     // KL <= N, so KL <= S / 2
+        load_row<LS, true>(g, G + row * KL, live ? KL : 0, t);     // KL <= N, so KL <= S / 2
         team.template forward<true>(g);
         if constexpr (DY) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) v[k] = cmul<false>(g[k], Q[k * F::M + t]);
             team.inverse(v);
-            if (live) store_row<LS, true>(v, dY + row * N, N, t, grow, KL, p, tanh_map, N);
+            y_fine &= store_row<LS>(v, dY + row * N, live ? N : 0, t, N);
         }
         if constexpr (DP) {
             load_row<LS, HALF>(v, Y + row * N, live ? N : 0, t);
@@ -507,6 +537,10 @@ fft_adjoint_kernel(const float* __restrict__ p, bool tanh_map, const float2* __r
         if (__syncthreads_or(!fine))
             direct_dp<LS>(G, Y, (long long)blockIdx.x * F::RT, sub, (long long)gridDim.x * F::RT, A,
                           N, KL, t, team.x, o);
+    }
+    if constexpr (DY) {
+        if (__syncthreads_or(!y_fine))
+            direct_rows<LS, true>(team.x, G, KL, dY, N, A, p, tanh_map, N, sub, t);
     }
 }
 
