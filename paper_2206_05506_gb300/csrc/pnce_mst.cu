@@ -322,15 +322,8 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
     const unsigned sbuf = (unsigned)__cvta_generic_to_shared(buf);
     const int teams = blockDim.x / M::TEAM;
     const long long stride = (long long)gridDim.x * teams * M::RT;
-    // Teams that start together load together and then add together.  Where a row is several
-    // microseconds of work (r >= 11) and each team has two or more, half of the teams start 2 us
-    // later: the other half's first rows still keep the memory busy, and from then on one half
-    // loads while the other adds.  us without / with: N = 2047, 4736 rows of 4 x 128 spread lags
-    // 31.7 / 29.8, 5473 rows of 1024 lags 32.0 / 29.6; N = 4095, 65536 rows of 2048 lags 552 /
-    // 545, fp16 615 / 606, 2737 rows 34.8 / 32.1, 32768 rows of 16 lags 177.5 / 174.2 (1.5 to 5 us
-    // are alike).  Shorter rows lose: N = 1023 fp16 1 %, N = 127 with 5 lags 5-13 %.
     if constexpr (R >= 11 && IO == ROWS && MODE != CODES) {
-        if (team >= teams / 2 && 2 * stride <= p.A) __nanosleep(2200);
+        if (team >= p.late_from) __nanosleep(2200);
     }
 
     for (long long row0 = ((long long)blockIdx.x * teams + team) * M::RT; row0 < p.A;
@@ -551,6 +544,29 @@ MstBatchKernel batch_kernel_of(int mode) {
     return mode == ROUND ? mst_batch_kernel<R, ROUND> : mst_batch_kernel<R, PLAIN>;
 }
 
+}  // namespace
+
+namespace pnce {
+
+// Teams that start together load together and then add together.  Where a row is several
+// microseconds of work (r >= 11), each team has two or more and a block has several, half of a
+// block's teams (r = 13: two of three) start 2 us later: the other half's first rows still keep the
+// memory busy, and from then on one half loads while the other adds.  us without / with: N = 2047,
+// 4736 rows of 4 x 128 spread lags 31.7 / 29.8, 5473 rows of 1024 lags 32.0 / 29.6; N = 4095, 65536
+// rows of 2048 lags 552 / 545, fp16 615 / 606, 2737 rows 34.8 / 32.1, 32768 rows of 16 lags 177.5 /
+// 174.2 (1.5 to 5 us are alike); N = 8191, 913 rows 43.9 / 41.8, 4000 rows 121.1 / 116.0 (one late
+// team of three: 43.2, 118.7).  Shorter rows lose: N = 1023 fp16 1 %, N = 127 with 5 lags 5-13 %.  A
+// block of one team (r = 14) has no other half, N = 16383, 304 rows 20.4 / 20.8, fp16, 608 rows 43.8 /
+// 45.2, nor do launches from host memory that keep one team per SM in flight (256 rows of N = 4095
+// 67.5 / 69.7).
+int mst_late_from(int r, int teams, bool two_rounds) {
+    return r >= 11 && teams > 1 && two_rounds ? teams / 2 : teams;
+}
+
+}  // namespace pnce
+
+namespace {
+
 template <int R>
 cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t s) {
     using M = Mst<R>;
@@ -573,6 +589,7 @@ cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t 
     const long long resident = sms * (per == m.block_teams ? m.blocks_per_sm : 1);
     if (grid > resident) grid = resident;
     if (p.in_flight && grid > (most + per - 1) / per) grid = (most + per - 1) / per;
+    p.late_from = pnce::mst_late_from(R, (int)per, 2 * grid * per * M::RT <= p.A);
     const int mode = p.operand ? CODES : p.dtype != PNCE_FP32_SIMT ? ROUND : PLAIN;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);

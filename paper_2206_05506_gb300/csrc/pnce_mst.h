@@ -40,6 +40,7 @@ struct MstLaunch {
     const uint16_t* tab = nullptr;
     const uint16_t* lagvec = nullptr;
     int lg_parts = 0;
+    int late_from = 0;           // teams of a block that start later: from this one on
     int N = 0;
     float invN = 0.f;
     unsigned magic_L = 0;
@@ -60,6 +61,9 @@ cudaError_t mst_setup(MstTables& m, const uint16_t* tab_dev, int N, int num_sms,
 // unless one of the switches that pick a tensor-core kernel (PNCE_TC_*) is set.
 bool mst_replaces_tc(const pnce_pilot* pilot);
 cudaError_t launch_mst(const MstTables& m, MstLaunch p, cudaStream_t s);
+// The first of a block's teams that starts late (teams: none does); two_rounds: every team has two
+// rows or more.
+int mst_late_from(int r, int teams, bool two_rounds);
 
 // Whether an estimate in a tensor-core dtype is one launch that rounds in registers.  Traced
 // calls keep the quantiser as a launch of its own, so that each step is timed; the results
