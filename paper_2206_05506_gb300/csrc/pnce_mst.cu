@@ -216,14 +216,23 @@ __device__ __forceinline__ void load_codes(const pnce::MstLaunch& p, long long r
 // Against one bit test and one addition per sample and lag (pnce_simt.cu), same sizes: r = 12,
 // 16 lags 253 -> 181, 8 lags 182 -> 174; r = 10, 16 lags 298 -> 178; r = 7, 8 lags 546 -> 218;
 // relative error 5.8-8.9e-8 -> 4.6-7.9e-8.
+// A batch's rows of as few lags take the same form, so that a request has the bits of an estimate
+// of its own in any mix; the other rows of the batch take the second pass.
 constexpr int few_cols(int r) { return r >= 11 ? 32 : r == 10 ? 16 : 8; }
+
+// P = 2^lg_parts: as many threads per column as a row's G allow, 32 at most
+__host__ __device__ constexpr int lg_parts_of(int cols, int G) {
+    int lg = 0;
+    while (lg < 5 && (cols << (lg + 1)) <= G) ++lg;
+    return lg;
+}
 
 // G (a power of two) values of one column: sum over t of (-1)^<ul, t> V_t, the P = 2^lgP
 // threads of the column taking every P-th each; the same on all P lanes.  row: V_t at
-// (t + rot) mod G.
+// (t + rot) mod G.  lanes: those of the warp that are here.
 template <int G>
 __device__ __forceinline__ float2 column_sum(const float2* row, int rot, unsigned ul, int part,
-                                             int lgP) {
+                                             int lgP, unsigned lanes) {
     const int n = G >> lgP;
     float2 acc[8];
 #pragma unroll
@@ -253,9 +262,24 @@ __device__ __forceinline__ float2 column_sum(const float2* row, int rot, unsigne
         for (int e = 0; e < d; ++e) acc[e] = __fadd2_rn(acc[e], acc[e + d]);
     float2 s = acc[0];
     for (int o = 1; o < (1 << lgP); o <<= 1)
-        s = __fadd2_rn(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o),
-                                      __shfl_xor_sync(0xffffffffu, s.y, o)));
+        s = __fadd2_rn(s, make_float2(__shfl_xor_sync(lanes, s.x, o),
+                                      __shfl_xor_sync(lanes, s.y, o)));
     return s;
+}
+
+// The columns of a row whose V_t[k] lie in the buffer, [k][(t + 4 k) mod G] (lanes of different
+// columns, 4 or more neighbours of each, mostly meet different bank pairs)
+template <int G, int LG>
+__device__ __forceinline__ void few_columns(const float2* buf, const uint16_t* u_of, int cols,
+                                            int lgP, int t, float scale, float2* h,
+                                            unsigned lanes) {
+    for (int c0 = 0; c0 < cols; c0 += G >> lgP) {
+        const int part = t & ((1 << lgP) - 1), c = c0 + (t >> lgP);
+        const unsigned u = u_of[c < cols ? c : 0], k = u >> LG;
+        const float2 w =
+            column_sum<G>(buf + k * G, (int)(4 * k), u & (G - 1), part, lgP, lanes);
+        if (h && part == 0 && c < cols) h[c] = make_float2(w.x * scale, w.y * scale);
+    }
 }
 
 // column k L + l holds lag k step + l
@@ -275,6 +299,10 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
     constexpr int E = M::E, G = M::G, LG = M::LG, LE = M::LE, S = M::S;
     extern __shared__ __align__(128) unsigned char mst_smem[];
     const int tid = threadIdx.x;
+    uint16_t u_tid = 0;                          // (its load overlaps those of the tables)
+    if constexpr (IO != ROWS) {
+        if (tid < few_cols(R)) u_tid = __ldg(p.lagvec + tid);      // a block has 32 threads or more
+    }
     const uint16_t* tab;
     if constexpr (M::TAB_SMEM) {
         const uint4* src = reinterpret_cast<const uint4*>(p.tab);
@@ -299,8 +327,10 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
             few_u[c] = (uint16_t)u;
             atomicOr(&few_rows[u >> LG >> 5], 1u << (u >> LG & 31));
         }
+    } else if constexpr (IO != ROWS) {
+        if (tid < few_cols(R)) few_u[tid] = u_tid;
     }
-    if constexpr (M::TAB_SMEM || FEW) __syncthreads();
+    if constexpr (M::TAB_SMEM || FEW || IO != ROWS) __syncthreads();
     const uint4* in_slot = reinterpret_cast<const uint4*>(tab);            // [E/8][G] x 8
     const uint4* out_slot = reinterpret_cast<const uint4*>(tab + S);       // [E/8][G] x 8
     const uint16_t* lag_slot = tab + 2 * S;                                // [N]
@@ -441,22 +471,35 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
         }
         butterflies<E, 1, E>(v);
         team_sync<M::TEAM>(team);                  // the buffer is read: reuse it
+        bool few = FEW, second = !FEW;             // forms of this row, and of its team's rows
         if constexpr (FEW) {
-            // V_t[k] at (t + 4 k) mod G of row k: lanes of different columns, 4 or more
-            // neighbours of each, mostly meet different bank pairs
             const unsigned rows0 = few_rows[0], rows1 = few_rows[1];
 #pragma unroll
             for (int k = 0; k < E; ++k)
                 if ((k < 32 ? rows0 : rows1) >> (k & 31) & 1)
                     buf[k * G + ((t + 4 * k) & (G - 1))] = v[k];
             team_sync<M::TEAM>(team);
-            for (int c0 = 0; c0 < cols; c0 += G >> p.lg_parts) {
-                const int part = t & ((1 << p.lg_parts) - 1), c = c0 + (t >> p.lg_parts);
-                const unsigned u = few_u[c < cols ? c : 0], k = u >> LG;
-                const float2 w = column_sum<G>(buf + k * G, (int)(4 * k), u & (G - 1), part, p.lg_parts);
-                if (h && part == 0 && c < cols) h[c] = make_float2(w.x * scale, w.y * scale);
+            few_columns<G, LG>(buf, few_u, cols, p.lg_parts, t, scale, h, 0xffffffffu);
+        } else if constexpr (IO != ROWS) {
+            few = cols <= few_cols(R);
+            if (M::RT == 1 ? few : __any_sync(0xffffffffu, few)) {
+                second = M::RT != 1 && __any_sync(0xffffffffu, !few);
+#pragma unroll
+                for (int k = 0; k < E; ++k) buf[k * G + ((t + 4 * k) & (G - 1))] = v[k];
+                team_sync<M::TEAM>(team);
+                // the rows of a warp may differ in their columns: each with its own lanes
+                const unsigned lanes =
+                    G < 32 ? ((1u << (G & 31)) - 1u) << ((tid & 31) & ~(G - 1)) : 0xffffffffu;
+                if (few)
+                    few_columns<G, LG>(buf, few_u, cols, lg_parts_of(cols, G), t, scale, h, lanes);
+                if (second) {                     // (read again: kept, they would not fit)
+#pragma unroll
+                    for (int k = 0; k < E; ++k) v[k] = buf[k * G + ((t + 4 * k) & (G - 1))];
+                    team_sync<M::TEAM>(team);
+                }
             }
-        } else {
+        }
+        if (second) {
 #pragma unroll
             for (int k = 0; k < E; ++k) {
                 const int s = k * G + t;
@@ -496,7 +539,7 @@ __device__ __forceinline__ void mst_rows(const pnce::MstLaunch& p, const pnce::M
                 }
             }
             team_sync<M::TEAM>(team);
-            if (h) {
+            if (h && !few) {
                 for (int c = t; c < cols; c += G) {
                     const int lag = IO != ROWS ? c : lag_of(p, c);
                     const float2 w = buf[lag_slot[lag]];
@@ -571,8 +614,7 @@ template <int R>
 cudaError_t launch_r(const pnce::MstTables& m, pnce::MstLaunch& p, cudaStream_t s) {
     using M = Mst<R>;
     const bool few = p.lagvec && !p.dd && !p.batch && p.lags.ldH <= few_cols(R);
-    p.lg_parts = 0;                              // threads per column, 32 at most
-    while (p.lg_parts < 5 && (p.lags.ldH << (p.lg_parts + 1)) <= M::G) ++p.lg_parts;
+    p.lg_parts = lg_parts_of(p.lags.ldH, M::G);
     // rows spread over the SMs first, then over the teams of a block
     const long long teams = (p.A + M::RT - 1) / M::RT;
     const long long sms = m.num_sms;
