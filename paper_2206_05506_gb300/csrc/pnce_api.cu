@@ -1,8 +1,10 @@
 // C ABI of libpnce: argument validation, handle / pilot objects and dispatch to the
 // kernels.  Nothing here computes the estimate; every step of it runs in the kernels.
+#include <cudaTypedefs.h>
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -510,21 +512,49 @@ pnce_status pnce_backward(pnce_handle* h, const float* p_dev, int pilot_map, con
 
 namespace {
 
+PFN_cuPointerGetAttribute_v4000 pointer_attribute_fn() {
+    static PFN_cuPointerGetAttribute_v4000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 12000, cudaEnableDefault,
+                                             &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(p);
+    });
+    return fn;
+}
+
 // The address at which the GPU reads and writes `bytes` bytes of page-locked host memory at p;
-// null if they are not page-locked or not 8-byte aligned.
+// null if they are not page-locked throughout (they may consist of several neighbouring ranges,
+// but a part between two of them that is not page-locked is no memory of the GPU's) or not 8-byte
+// aligned.
 void* host_mapped(const void* p, size_t bytes) {
-    cudaPointerAttributes at{}, last{};
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();                      // unknown pointer
-        return nullptr;
+    const PFN_cuPointerGetAttribute_v4000 attribute = pointer_attribute_fn();
+    const uintptr_t first = (uintptr_t)p, end = first + bytes;
+    char* mapped = nullptr;
+    if (!attribute) return nullptr;
+    for (uintptr_t q = first; q < end;) {
+        cudaPointerAttributes at{};
+        CUdeviceptr start = 0;
+        size_t size = 0;
+        if (cudaPointerGetAttributes(&at, reinterpret_cast<void*>(q)) != cudaSuccess) {
+            cudaGetLastError();                  // unknown pointer
+            return nullptr;
+        }
+        if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+        if (q == first) mapped = static_cast<char*>(at.devicePointer);
+        if (static_cast<char*>(at.devicePointer) != mapped + (q - first)) return nullptr;
+        // the range of the driver that holds q
+        const CUdeviceptr dq = (CUdeviceptr)(uintptr_t)at.devicePointer;
+        if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, dq) != CUDA_SUCCESS ||
+            attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, dq) != CUDA_SUCCESS ||
+            dq < start || dq - start >= size)
+            return nullptr;
+        q += size - (size_t)(dq - start);
     }
-    if (at.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !at.devicePointer ||
-        static_cast<char*>(last.devicePointer) - static_cast<char*>(at.devicePointer) !=
-            (ptrdiff_t)bytes - 1 ||
-        ((uintptr_t)at.devicePointer & 7u))
-        return nullptr;
-    return at.devicePointer;
+    return ((uintptr_t)mapped & 7u) ? nullptr : mapped;
 }
 
 // Host pipeline layout: frames go through in chunks of fc frames, kPnceHostSlots slots of
