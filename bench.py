@@ -697,6 +697,36 @@ def run_reference(args, w):
     print(json.dumps(line), flush=True)
 
 
+def kernels_of(step):
+    """Kernel launches of one call of step(), from the nodes of a captured graph."""
+    import ctypes
+
+    import torch
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        step()
+    cu, graph, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes, kind = (ctypes.c_void_p * n.value)(), ctypes.c_int(0)
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kernels = 0
+    for node in nodes:
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kernels += kind.value == 0               # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
+def max_frame_nmse(a, b):
+    """The largest NMSE of a against b over the frames (first dimension), in 64 bits."""
+    import torch
+    worst = 0.0
+    for f in range(0, a.shape[0], 32):
+        x, y = a[f:f + 32].to(torch.complex128), b[f:f + 32].to(torch.complex128)
+        num, den = ((z.abs() ** 2).flatten(1).sum(1) for z in (x - y, y))
+        worst = max(worst, float((num / den).max()))
+    return worst
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -800,7 +830,8 @@ def main():
     clk = clocks.stop()
     total_ms = max_over_ranks(e_start.elapsed_time(e_end), world, dev)
     assert pk.get_status(dev) == 0
-    launches = args.steps            # one per estimate (m-sequence pilot, no switch set)
+    step_kernels = kernels_of(step)  # counted in a capture of the same call
+    launches = args.steps * step_kernels
 
     taps_per_step = F * M * K * L
     value = taps_per_step * args.steps * world / (total_ms / 1e3)
@@ -822,7 +853,13 @@ def main():
         pk.trace_enable(False, dev)
         del os.environ["PNCE_TC_FORCE"]
         tc_ms = {kind: float(np.mean(v)) for kind, v in tc_ms.items()}
+        H_tc = H.clone()
         step()                       # H: the product call's result again
+        # the result that the tensor cores' rate belongs to, against the product call's, which the
+        # oracle checks below
+        tc_nmse = max_frame_nmse(H_tc, H)
+        assert tc_nmse <= 1e-6, tc_nmse
+        del H_tc
 
     # ---- end to end through the host-buffer entry point
     H_pin = torch.empty((F, M, K, L), dtype=torch.complex64, pin_memory=True)
@@ -867,6 +904,7 @@ def main():
         roof["tensor_cores"] = {"kernel": "tc_corr_kernel", "ms_per_launch": tc_ms["correlate"],
                                 "quantize_ms": tc_ms["quantize"], "achieved": tflops,
                                 "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
+                                "max_frame_nmse_vs_estimate": tc_nmse,
                                 "traffic": traffic_from_profile(w.name, dt, F)}
 
     # ---- CPU baseline (FP64 oracle) on a frame sample, plus accuracy of those frames.  It
@@ -941,7 +979,7 @@ def main():
         "config": {"workload": w.name, "frames": F, "M": M, "N": N, "K": K, "L": L,
                    "snr_db": list(w.snr_db), "parallelism": f"frames x{world}",
                    "l2": f"inputs larger than L2 ({Y.numel() * 8 / 1e9:.2f} GB Y per step)"},
-        "breakdown_ms": {"estimate_per_launch": kern_ms, "launches_per_step": 1},
+        "breakdown_ms": {"estimate_per_launch": kern_ms, "launches_per_step": step_kernels},
         "roofline": roof,
         "e2e": {"value": e2e_value, "unit": "taps/s",
                 "h2d_bytes_per_step": int(Y_pin.numel() * 8),
