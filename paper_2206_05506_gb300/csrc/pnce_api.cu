@@ -512,16 +512,16 @@ pnce_status pnce_backward(pnce_handle* h, const float* p_dev, int pilot_map, con
 
 namespace {
 
-PFN_cuPointerGetAttribute_v4000 pointer_attribute_fn() {
-    static PFN_cuPointerGetAttribute_v4000 fn = nullptr;
+PFN_cuPointerGetAttributes_v7000 pointer_attributes_fn() {
+    static PFN_cuPointerGetAttributes_v7000 fn = nullptr;
     static std::once_flag once;
     std::call_once(once, [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 12000, cudaEnableDefault,
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 12000, cudaEnableDefault,
                                              &q) == cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(p);
+            fn = reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(p);
     });
     return fn;
 }
@@ -531,30 +531,29 @@ PFN_cuPointerGetAttribute_v4000 pointer_attribute_fn() {
 // but a part between two of them that is not page-locked is no memory of the GPU's) or not 8-byte
 // aligned.
 void* host_mapped(const void* p, size_t bytes) {
-    const PFN_cuPointerGetAttribute_v4000 attribute = pointer_attribute_fn();
+    const PFN_cuPointerGetAttributes_v7000 attributes = pointer_attributes_fn();
     const uintptr_t first = (uintptr_t)p, end = first + bytes;
-    char* mapped = nullptr;
-    if (!attribute) return nullptr;
+    uintptr_t mapped = 0;
+    if (!attributes) return nullptr;
     for (uintptr_t q = first; q < end;) {
-        cudaPointerAttributes at{};
-        CUdeviceptr start = 0;
+        // all zero for a pointer that the driver does not know
+        unsigned type = 0, managed = 0;
+        CUdeviceptr dev = 0, start = 0;
         size_t size = 0;
-        if (cudaPointerGetAttributes(&at, reinterpret_cast<void*>(q)) != cudaSuccess) {
-            cudaGetLastError();                  // unknown pointer
+        CUpointer_attribute what[5] = {
+            CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+            CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+            CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+        void* value[5] = {&type, &managed, &dev, &start, &size};
+        if (attributes(5, what, value, (CUdeviceptr)q) != CUDA_SUCCESS ||
+            type != CU_MEMORYTYPE_HOST || managed || !dev)
             return nullptr;
-        }
-        if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
-        if (q == first) mapped = static_cast<char*>(at.devicePointer);
-        if (static_cast<char*>(at.devicePointer) != mapped + (q - first)) return nullptr;
-        // the range of the driver that holds q
-        const CUdeviceptr dq = (CUdeviceptr)(uintptr_t)at.devicePointer;
-        if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, dq) != CUDA_SUCCESS ||
-            attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, dq) != CUDA_SUCCESS ||
-            dq < start || dq - start >= size)
-            return nullptr;
-        q += size - (size_t)(dq - start);
+        if (q == first) mapped = (uintptr_t)dev;
+        if ((uintptr_t)dev != mapped + (q - first)) return nullptr;
+        if (q < start || q - start >= size) return nullptr;
+        q = (uintptr_t)start + size;             // the next range
     }
-    return ((uintptr_t)mapped & 7u) ? nullptr : mapped;
+    return (mapped & 7u) ? nullptr : reinterpret_cast<void*>(mapped);
 }
 
 // Host pipeline layout: frames go through in chunks of fc frames, kPnceHostSlots slots of
