@@ -104,8 +104,10 @@ pnce_status pnce_get_status(pnce_handle* h, void* stream);
 /*
  * Pilot table (Sec. II-A: the m-sequence pilot, Eq. 1).  bits_host: ceil(N/32) uint32
  * words, bit n of the sequence in word n/32 at bit n%32 (LSB first).  The library
- * uploads a wrapped copy (bit t = bit (t mod N)) to device memory once; the call is
- * synchronous.  N in [2, 2^24).
+ * uploads a wrapped copy (bit t = bit (t mod N)) to device memory once, and for an
+ * m-sequence of 127 <= N <= 16383 the tables of its fast transform, which the host builds
+ * (17 us at N = 127, 0.28 ms at 4095, 1.3 ms at 16383; 7 to 22 us otherwise): keep the
+ * pilot over the calls that use it.  Synchronous.  N in [2, 2^24).
  */
 pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, pnce_pilot** out);
 pnce_status pnce_pilot_destroy(pnce_pilot* p);
@@ -201,7 +203,8 @@ typedef enum {
 /*
  * Estimate with a real-valued pilot (float32 [N], device) in place of the +-1 sequence:
  * H = (1/N) sum_n Y[n] p[(n - j) mod N], FP32 on the CUDA cores (by FFT for N >= 84 up to
- * N + K*L - 1 = 4096; rows that hold or reach infinities are summed directly).  With PNCE_PILOT_TANH
+ * N + K*L - 1 = 4096, with errors relative to the row's norm; outputs of rows that hold or
+ * reach infinities are summed directly).  With PNCE_PILOT_TANH
  * the argument is theta and p = tanh(theta) is formed inside the kernel: the forward of
  * the relaxed pilot used for end-to-end pilot optimisation.
  */
@@ -217,7 +220,8 @@ pnce_status pnce_estimate_real_pilot(pnce_handle* h, const float* pilot_dev, int
  * and with PNCE_PILOT_TANH, dpilot_dev is the gradient with respect to theta,
  * dp[q] * (1 - tanh(theta[q])^2).  The pilot sum is reduced deterministically in two
  * stages through workspace_dev (pnce_backward_workspace_size bytes), so repeated calls
- * give identical bits.
+ * give identical bits.  By FFT from 128 lags on up to N + K*L - 1 = 4096: errors are then
+ * relative to the row's norm (1.6e-7 to 2e-7) also where few lags of G are not zero.
  */
 size_t pnce_backward_workspace_size(int F, int M, int N, int K, int L);
 pnce_status pnce_backward(pnce_handle* h, const float* pilot_dev, int pilot_map,
@@ -257,12 +261,11 @@ pnce_status pnce_estimate_host(pnce_handle* h, const pnce_pilot* pilot, const vo
  * "pnce.<kind>" (always on; a no-op unless a profiler is attached).
  * pnce_trace_enable creates the events on first use (allocates host and event resources,
  * not device memory) and clears the record; pnce_trace_read waits for the recorded kernels,
- * (traced calls quantise and correlate in two launches even where an untraced one takes
- * one; the results are the same bits)
- * returns up to max_entries (kind, milliseconds) pairs -- kind 0 quantiser, 1 tensor-core
- * correlation, 2 FP32 SIMT correlation, 3 fast m-sequence transform, 4 adjoint (dY and
- * dp together) -- in launch order, and
- * clears the record.  Do not enable it while capturing a CUDA graph.
+ * returns up to max_entries (kind, milliseconds) pairs -- kind 0 quantiser, 1 correlation of a
+ * tensor-core dtype, 2 FP32 correlation, 3 pnce_estimate_fmt, 4 adjoint (dY and dp together) --
+ * in launch order, and clears the record.  A traced call of a tensor-core dtype quantises and
+ * correlates in two launches even where an untraced one takes one; the results are the same
+ * bits.  Do not enable it while capturing a CUDA graph.
  */
 pnce_status pnce_trace_enable(pnce_handle* h, int on);
 pnce_status pnce_trace_read(pnce_handle* h, int* kinds, float* ms, int max_entries, int* count);
@@ -298,13 +301,15 @@ pnce_status pnce_trace_read(pnce_handle* h, int* kinds, float* ms, int max_entri
  * no request covers are estimated from zeros or whatever the workspace holds, and
  * discarded.  workspace_dev: 256-byte aligned, pnce_grouped_workspace_size(rows, N,
  * kl_max, dtype) bytes (0 for invalid shapes).  Enqueues on `stream`, each kernel a
- * programmatic dependent of the one before it: a table / row-map kernel, then for the
- * tensor-core dtypes the quantiser (reading each row from its request's Y), the
- * correlation and a scatter into the requests' H; for FP32 with an m-sequence pilot the
- * fast transform, reading from and writing into the requests' buffers; with other pilots
- * and kl_max > 32 the SIMT correlation reading the rows from the requests' Y (after a row gather into the
- * workspace when kl_max > 256) and writing each row's lags into its request's H; for
- * FP32 with kl_max <= 32 a row gather, the correlation and a scatter.  Allocates nothing.
+ * programmatic dependent of the one before it: a table / row-map kernel, then with an
+ * m-sequence pilot (127 <= N <= 16383) the fast transform, reading from and writing into the
+ * requests' buffers; with other pilots, for the tensor-core dtypes the quantiser (reading
+ * each row from its request's Y), the correlation and a scatter into the requests' H; for
+ * FP32 with kl_max > 32 the SIMT correlation reading the rows from the requests' Y (after a
+ * row gather into the workspace when kl_max > 256) and writing each row's lags into its
+ * request's H; for FP32 with kl_max <= 32 a row gather, the correlation and a scatter.  Each
+ * request gets the bits that pnce_estimate gives it alone, except, in FP32 with such other
+ * pilots, requests of at most 32 lags in a batch of more.  Allocates nothing.
  */
 typedef struct {
     const void* Y;          /* complex64 [M][N] */
