@@ -291,7 +291,7 @@ pnce_status pnce_pilot_create(pnce_handle* h, const uint32_t* bits_host, int N, 
         return PNCE_ENOMEM;
     }
     const uint16_t* tab = reinterpret_cast<const uint16_t*>(p->ext_bits_dev + bits_bytes / 4);
-    if (cudaMemcpy(p->ext_bits_dev, ext.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (pnce::upload(p->ext_bits_dev, ext.data(), bytes) != cudaSuccess ||
         (mst_bytes && pnce::mst_setup(p->mst, tab, N, h->num_sms, h->max_smem_optin) != cudaSuccess)) {
         cudaFree(p->ext_bits_dev);
         delete p;

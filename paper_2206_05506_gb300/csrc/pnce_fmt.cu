@@ -169,7 +169,7 @@ pnce_status pnce_fmt_create(pnce_handle* h, const uint32_t* bits_host, int N, pn
         delete f;
         return PNCE_ENOMEM;
     }
-    if (cudaMemcpy(f->tab_dev, tab.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (pnce::upload(f->tab_dev, tab.data(), bytes) != cudaSuccess ||
         (mst && pnce::mst_setup(f->mst, f->tab_dev, N, h->num_sms, h->max_smem_optin) != cudaSuccess)) {
         cudaFree(f->tab_dev);
         delete f;

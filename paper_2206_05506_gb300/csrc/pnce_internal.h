@@ -85,6 +85,14 @@ struct TraceScope {
 }  // namespace pnce
 
 namespace pnce {
+// Copies pageable memory to the device and waits until it is there.  cudaMemcpy alone may return
+// when the bytes are staged, and work on a non-blocking stream (a serving slot's, where the first
+// batch may follow at once) does not wait for the copy.
+inline cudaError_t upload(void* dev, const void* host, size_t bytes) {
+    const cudaError_t e = cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamLegacy);
+}
+
 // Fast m-sequence transform of one pilot (pnce_mst.cu): its tables on the device (null: the
 // pilot is no m-sequence of a supported degree) and the launch shape that fits an SM.
 struct MstTables {
